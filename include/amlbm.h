@@ -69,7 +69,8 @@ extern "C" {
 /* How the force F enters the collision (Sec. II.B; Sec. IV.1 compares the two). */
 #define AMLBM_FORCE_SHIFT 0 /* Shan-Chen velocity shift: f^eq at u^eq = (rho u + tau F)/rho */
 #define AMLBM_FORCE_GUO 1   /* Guo, Zheng & Shi (2002): f^eq at u, plus (1 - 1/(2 tau)) times
-                               W_i [3 (c_i - u) + 9 (c_i . u) c_i] . F; fused schedule only, no adjoint */
+                               W_i [3 (c_i - u) + 9 (c_i . u) c_i] . F; not on a requested split
+                               schedule, no adjoint */
 
 /* Lower radial boundary. */
 #define AMLBM_RLO_AXIS 0  /* the axis r = 0, half a spacing below row 0 (r_off = 0) */
@@ -164,8 +165,8 @@ size_t amlbm_workspace_bytes(int Nz, int Nr, int storage);
  * shift, g_z = 0, rho_ref = 1, periodic z on the axis).  Requires Nz >= 1, Nr >= 4,
  * tau > 1/2, rho0 > 0, G >= -6.5 (the paper's stability limit is G >= -6,
  * Sec. II.D); z walls need Nz >= 4, inlet or outlet rows Nr >= 6.  A bounded
- * domain (z walls, inlet or outlet) runs on the fused schedule only and has no
- * adjoint (AMLBM_EINVAL).  cuda_stream is a cudaStream_t.  workspace: see
+ * domain (z walls, inlet or outlet) runs on the library's own choice or the fused
+ * schedule and has no adjoint (AMLBM_EINVAL).  cuda_stream is a cudaStream_t.  workspace: see
  * "Memory and ownership". */
 int amlbm_create(int Nz, int Nr, double tau, double G, double rho0, const amlbm_bc* bc,
                  void* cuda_stream, void* workspace, size_t workspace_bytes, amlbm_ctx** out);
@@ -329,7 +330,10 @@ typedef struct amlbm_instance {
 /* How a timestep is launched.  FUSED: one kernel per tile computes the whole
  * update, recomputing forces and velocities on a 3-site halo.  SPLIT: a force
  * kernel writes u and u^eq per site, then a collide-stream kernel reads them with
- * a halo (less recomputation, 16 or 32 more bytes per site through L2).  PAIR:
+ * a halo (less recomputation, 16 or 32 more bytes per site through L2); for FP64
+ * the force kernel also collides, in place, and nearly nothing is recomputed: the
+ * library's choice for every FP64 lattice, the bounded ones too, which a caller
+ * cannot request it for.  PAIR:
  * the fused update with two adjacent z-sites per thread (vector loads and
  * stores, stencil taps shared by the pair); it takes periodic lattices on the
  * axis with an even Nz, a free-slip or no-slip outer wall, the source at the

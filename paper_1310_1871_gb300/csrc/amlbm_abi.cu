@@ -107,29 +107,46 @@ bool all_pair_ok(const std::vector<amlbm_instance>& inst) {
   return true;
 }
 
-// Schedule and tile when the caller gives none (fastest on the 64-drop sweep on
-// GB300): the FP32-arithmetic forms take the pair schedule where every lattice
-// allows it (else the fused one), with the first tile of a preference list that
-// still gives every SM two CTAs over the whole batch; the FP64 form, bound by
-// FP64 arithmetic, takes the split schedule (less recomputation).
+// Tiles of tz x tr sites over all lattices.
+long long count_tiles(const std::vector<amlbm_instance>& inst, int tz, int tr) {
+  long long n = 0;
+  for (const auto& I : inst) n += (long long)((I.Nz + tz - 1) / tz) * ((I.Nr + tr - 1) / tr);
+  return n;
+}
+
+// Schedule and tile when the caller gives none.
+//
+// FP64: the two kernels of amlbm_step_split64.cu, on the largest tile that still keeps
+// the 152 SMs busy.  Measured (us per step on 8 x 4 / 16 x 8 / 32 x 8 / 32 x 16 tiles):
+// 64 x 32 11.2 / 16.5 / 22.4 / 37.3 (the recomputing kernels before: 38); 192 x 96 17.8 /
+// 16.1 / 22.5 / 37.7; 256 x 128 26.1 / 24.2 / 23.0 / 38.3; 512 x 256 90 / 68 / 68.0 / 66.5;
+// 1024 x 512 338 / 250 / 227 / 218 (before: 394); 330,400 sites in 25 lattices 217 / 168 /
+// 158.5 / 164.5.
+//
+// FP32 arithmetic: the pair schedule where every lattice allows it, else the fused
+// one, with the first tile of a preference list that still gives every SM two CTAs
+// over the whole batch.
 void pick_tile(int storage, const std::vector<amlbm_instance>& inst, int* sched, int* tz, int* tr) {
-  static const int pref64[][2] = {{32, 16}, {32, 8}, {32, 8}};
-  static const int pref64f[][2] = {{32, 8}, {32, 8}, {32, 8}};  // fused, for bounded lattices
+  if (storage == AMLBM_STORE_F64) {
+    static const struct { int tz, tr, least; } pref64[] = {{32, 16, 912}, {32, 8, 96}, {16, 8, 128}, {8, 4, 0}};
+    *sched = amlbm::SCHED_SPLIT;
+    for (const auto& t : pref64) {
+      *tz = t.tz;
+      *tr = t.tr;
+      if (count_tiles(inst, t.tz, t.tr) >= t.least) return;
+    }
+  }
   static const int pref32[][2] = {{26, 16}, {64, 8}, {32, 8}};
   static const int prefpair[][2] = {{64, 24}, {40, 24}, {24, 16}};
-  bool any_bounded = false;
-  for (const auto& I : inst) any_bounded = any_bounded || bounded(I.bc);
-  const bool f64 = storage == AMLBM_STORE_F64;
-  const bool pair = !f64 && all_pair_ok(inst);
-  const int(*pref)[2] = f64 ? (any_bounded ? pref64f : pref64) : pair ? prefpair : pref32;
-  *sched = f64 && !any_bounded ? amlbm::SCHED_SPLIT : pair ? amlbm::SCHED_PAIR : amlbm::SCHED_FUSED;
+  const bool pair = all_pair_ok(inst);
+  const int(*pref)[2] = pair ? prefpair : pref32;
+  *sched = pair ? amlbm::SCHED_PAIR : amlbm::SCHED_FUSED;
   for (int c = 0; c < 3; ++c) {
-    const int z = pref[c][0], r = pref[c][1];
-    long long tiles = 0;
-    for (const auto& I : inst) tiles += (long long)((I.Nz + z - 1) / z) * ((I.Nr + r - 1) / r);
-    if (tiles >= 2 * 152) { *tz = z; *tr = r; return; }
+    *tz = pref[c][0];
+    *tr = pref[c][1];
+    if (count_tiles(inst, *tz, *tr) >= 2 * 152) return;
   }
-  *sched = f64 && !any_bounded ? amlbm::SCHED_SPLIT : amlbm::SCHED_FUSED;
+  *sched = amlbm::SCHED_FUSED;
   *tz = 32;
   *tr = 8;
 }
@@ -200,17 +217,6 @@ struct Layout {
   long long sumN = 0, sumNz = 0;
 };
 
-// Tile of the read-back kernel: a pair batch reads back with the pair schedule's
-// kernel on its step tile, every other batch with the fused read-back (rb_tile()).
-void rb_tiling(int storage, int sched, int tz, int tr, int* rz, int* rr) {
-  if (sched == amlbm::SCHED_PAIR) {
-    *rz = tz;
-    *rr = tr;
-  } else {
-    amlbm::rb_tile(storage, rz, rr);
-  }
-}
-
 Layout make_layout(const std::vector<amlbm_instance>& inst, int storage, int tz, int tr, int sched) {
   Layout L;
   size_t o = 0;
@@ -219,7 +225,7 @@ Layout make_layout(const std::vector<amlbm_instance>& inst, int storage, int tz,
   for (const auto& I : inst) {
     L.ntiles += ((I.Nz + tz - 1) / tz) * ((I.Nr + tr - 1) / tr);
     int rz, rr;
-    rb_tiling(storage, sched, tz, tr, &rz, &rr);
+    amlbm::rb_tile(storage, sched, tz, tr, &rz, &rr);
     L.rb_ntiles += ((I.Nz + rz - 1) / rz) * ((I.Nr + rr - 1) / rr);
     L.maxN = std::max(L.maxN, I.Nz * I.Nr);
     L.maxNz = std::max(L.maxNz, I.Nz);
@@ -345,7 +351,7 @@ int batch_build(const std::vector<amlbm_instance>& inst, const amlbm_tune* tune,
                   "no-slip wall and the source at the departure site");
     if (sched == AMLBM_SCHED_SPLIT)
       for (const auto& I : inst)
-        if (bounded(I.bc))
+        if (bounded(I.bc))  // the FP64 kernels would take them; the documented choice is refused all the same
           return fail(AMLBM_EINVAL,
                       "the split schedule takes periodic lattices on the axis with the velocity shift only");
     if (!tz && !tr) {
@@ -417,7 +423,7 @@ int batch_build(const std::vector<amlbm_instance>& inst, const amlbm_tune* tune,
     d.tiles_r = (I.Nr + tr - 1) / tr;
     d.tile_base = (int)tiles.size();
     int rz, rr;
-    rb_tiling(storage, sched, tz, tr, &rz, &rr);
+    amlbm::rb_tile(storage, sched, tz, tr, &rz, &rr);
     d.rb_tiles_z = (I.Nz + rz - 1) / rz;
     d.rb_tiles_r = (I.Nr + rr - 1) / rr;
     d.rb_tile_base = (int)rb_tiles.size();
@@ -426,10 +432,12 @@ int batch_build(const std::vector<amlbm_instance>& inst, const amlbm_tune* tune,
     d.rho0 = I.rho0;
     d.gz = I.bc.g_z;
     d.rho_ref = I.bc.rho_ref;
-    const double k[12] = {I.tau, 1.0 / I.tau, -I.G, -I.G / 18.0, I.bc.g_z, I.rho0, 1.0 / I.rho0,
+    const double k[amlbm::kStepConstants] = {I.tau, 1.0 / I.tau, -I.G, -I.G / 18.0, I.bc.g_z, I.rho0, 1.0 / I.rho0,
                           (I.tau - 0.5) / 3.0, I.bc.rho_ref, I.bc.r_off + 0.5,
-                          I.bc.wall_r == AMLBM_WALL_OUTLET ? I.bc.rho_out : 1.0, 1.0 - 0.5 / I.tau};
-    for (int c = 0; c < 12; ++c) {
+                          I.bc.wall_r == AMLBM_WALL_OUTLET ? I.bc.rho_out : 1.0, 1.0 - 0.5 / I.tau,
+                          -I.G / 36.0, -I.G / (18.0 * 1296.0), 1.0 - 1.0 / I.tau, 1.0 / (9.0 * I.tau),
+                          (I.tau - 0.5) / 36.0};
+    for (int c = 0; c < amlbm::kStepConstants; ++c) {
       d.k64[c] = k[c];
       d.k32[c] = (float)k[c];
     }
@@ -484,7 +492,9 @@ int batch_build(const std::vector<amlbm_instance>& inst, const amlbm_tune* tune,
   }
   // the allocation-free diagnostics' scratch: looked up now, in a call that
   // allocates anyway (its failure surfaces at that entry point, not here)
-  amlbm::noalloc_prepare(storage);
+  int rz, rr;
+  amlbm::rb_tile(storage, sched, tz, tr, &rz, &rr);
+  amlbm::noalloc_prepare(storage, rz, rr);
   // the pair read-back's code, loaded now for the same reason (its first use
   // may be an allocation-free diagnostics call)
   if (sched == amlbm::SCHED_PAIR) amlbm::readback_pair_preload(storage, tz, tr);
@@ -550,7 +560,7 @@ cudaError_t launch_readback(amlbm_batch* b, int nt, int toff) {
     return amlbm::launch_readback_pair(b->storage, b->tz, b->tr, b->d_desc, b->d_rb_tiles, nt, toff, b->parity,
                                        b->stream);
   int rz, rr;
-  amlbm::rb_tile(b->storage, &rz, &rr);
+  amlbm::rb_tile(b->storage, b->sched, b->tz, b->tr, &rz, &rr);
   return amlbm::launch_macro(b->storage, rz, rr, b->d_desc, b->d_rb_tiles, nt, toff, b->parity, b->stream);
 }
 

@@ -529,7 +529,7 @@ namespace {
 
 struct AdjLayout {
   size_t total = 0;
-  size_t ckpt = 0, seg = 0, lam = 0, inter = 0, mu = 0, arr = 0, drp = 0, acc = 0, rho0 = 0,
+  size_t ckpt = 0, seg = 0, lam = 0, inter = 0, fstar = 0, mu = 0, arr = 0, drp = 0, acc = 0, rho0 = 0,
          red = 0, descs = 0, tiles = 0;
   int nck = 0, nseg = 0, ntiles = 0, nred = 0;
   int nbuf = 1;            // segment buffers: two when there are several segments
@@ -548,7 +548,9 @@ AdjLayout adj_layout(const amlbm::CtxInfo& ci, const amlbm_adjoint_problem& p) {
   L.nseg = std::min(p.ckpt_every, p.T);
   L.nbuf = L.nck > 1 ? 2 : 1;
   L.state_elems = 10 * plane;
-  L.ntiles = ((ci.Nz + 31) / 32) * ((ci.Nr + 7) / 8);
+  int tz, tr;
+  amlbm::inter_tile(ci.storage, ci.Nz, ci.Nr, &tz, &tr);
+  L.ntiles = ((ci.Nz + tz - 1) / tz) * ((ci.Nr + tr - 1) / tr);
   L.nred = std::min(1024, (ci.Nz * ci.Nr + 255) / 256);
   size_t o = 0;
   auto take = [&](size_t b) { const size_t a = o; o = al(o + b); return a; };
@@ -557,6 +559,7 @@ AdjLayout adj_layout(const amlbm::CtxInfo& ci, const amlbm_adjoint_problem& p) {
   L.seg = take((size_t)L.nbuf * (L.nseg + 1) * L.state_elems * cb);
   L.lam = take(2 * 9 * plane * cb);
   L.inter = take((size_t)L.nbuf * L.nseg * amlbm::I_COUNT * plane * cb);
+  L.fstar = take(ci.storage == AMLBM_STORE_F64 ? 9 * plane * cb : 0);
   L.mu = take(9 * plane * cb);
   L.arr = take((size_t)kAdjArrays * plane * cb);
   L.drp = take((size_t)(ci.Nr + 4) * ci.host.P * cb);
@@ -637,7 +640,7 @@ int run(amlbm_ctx* ctx, const amlbm_adjoint_problem* p, void* ws, size_t ws_byte
     const size_t SB = L.state_elems * sizeof(C), FB = 9 * plane * sizeof(C), PB = plane * sizeof(C);
     void* fcur;
     void* pcur;
-    int pitch;
+    int pitch, tz, tr;
 
     DropMap M;
     std::memset(&M, 0, sizeof(M));
@@ -683,15 +686,16 @@ int run(amlbm_ctx* ctx, const amlbm_adjoint_problem* p, void* ws, size_t ws_byte
                                         lam[0]);
       ADJ_CK(cudaGetLastError());
     }
-    // descriptors of the segment slots (tile 32 x 8): descriptor q of buffer b
+    // descriptors of the segment slots (tiled by inter_tile): descriptor q of buffer b
     // steps slot q of that buffer into slot q + 1
     {
       std::vector<InstDesc> d((size_t)L.nbuf * L.nseg, ci.host);
+      inter_tile(ci.storage, Nz, Nr, &tz, &tr);
       for (int b = 0; b < L.nbuf; ++b)
         for (int q = 0; q < L.nseg; ++q) {
           InstDesc& x = d[(size_t)b * L.nseg + q];
-          x.tiles_z = (Nz + 31) / 32;
-          x.tiles_r = (Nr + 7) / 8;
+          x.tiles_z = (Nz + tz - 1) / tz;
+          x.tiles_r = (Nr + tr - 1) / tr;
           x.tile_base = 0;
           C* sb = seg + (size_t)b * (L.nseg + 1) * L.state_elems;
           for (int h = 0; h < 2; ++h) {
@@ -734,8 +738,8 @@ int run(amlbm_ctx* ctx, const amlbm_adjoint_problem* p, void* ws, size_t ws_byte
       // the next state and the intermediates of the state it starts from).
       auto recompute = [&](int len, int b, cudaStream_t st) -> cudaError_t {
         for (int q = 0; q < len; ++q) {
-          const cudaError_t e = launch_step_inter(ci.storage, 32, 8, d_seg + (size_t)b * L.nseg + q, d_tiles,
-                                                  L.ntiles, inter_of(b) + q * iseg, plane, st);
+          const cudaError_t e = launch_step_inter(ci.storage, tz, tr, d_seg + (size_t)b * L.nseg + q, d_tiles, L.ntiles,
+                                                  inter_of(b) + q * iseg, plane, base + L.fstar, st);
           if (e != cudaSuccess) return e;
         }
         return cudaSuccess;

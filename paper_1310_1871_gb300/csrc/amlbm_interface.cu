@@ -144,8 +144,10 @@ extern "C" int amlbm_flat_interface(double G, double tau, double rho0, int axisy
   d.psi[0] = ci.host.psi[ci.parity];
   d.f[1] = ci.host.f[ci.parity ^ 1];
   d.psi[1] = ci.host.psi[ci.parity ^ 1];
+  int itz, itr;
+  amlbm::inter_tile(storage, 1, n, &itz, &itr);
   d.tiles_z = 1;
-  d.tiles_r = (n + 7) / 8;
+  d.tiles_r = (n + itr - 1) / itr;
   d.tile_base = 0;
   const int ntiles = d.tiles_r;
   const size_t cb = storage == AMLBM_STORE_F64 ? 8 : 4;
@@ -164,8 +166,9 @@ extern "C" int amlbm_flat_interface(double G, double tau, double rho0, int axisy
   e = cudaMemcpyAsync(B.p[0], &d, sizeof(InstDesc), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(B.p[1], 0, ntiles * sizeof(int), s);
   if (e == cudaSuccess)
-    e = amlbm::launch_step_inter(storage, 32, 8, static_cast<const InstDesc*>(B.p[0]),
-                                 static_cast<const int*>(B.p[1]), ntiles, B.p[2], plane, s);
+    e = amlbm::launch_step_inter(storage, itz, itr, static_cast<const InstDesc*>(B.p[0]), 
+                                 static_cast<const int*>(B.p[1]), ntiles, B.p[2], plane, d.f[0],
+                                 s);  // that state is not needed any more
   if (e == cudaSuccess) {
     const double r0 = 0.5;
     if (storage == AMLBM_STORE_F64)

@@ -10,6 +10,9 @@
 
 namespace amlbm {
 
+// Slots of InstDesc::k64 / k32.
+constexpr int kStepConstants = 17;
+
 // One lattice of a batch as the kernels see it.  Populations are stored as
 // [9][Nr][P] (z contiguous, row pitch P elements) and psi as [Nr][P]; both come
 // in two copies (ping-pong) selected by the batch-wide parity.
@@ -27,13 +30,16 @@ struct InstDesc {
   // the constants of the step, computed on the host in FP64 and also held
   // rounded to FP32 (kernels read them without conversion or division):
   // tau, 1/tau, -G, -G/18, g_z, rho0, 1/rho0, (tau - 1/2)/3, rho_ref,
-  // the radius of row 0 (r_off + 1/2), the outlet density and 1 - 1/(2 tau)
-  double k64[12];
-  float k32[12];
+  // the radius of row 0 (r_off + 1/2), the outlet density, 1 - 1/(2 tau), and for
+  // the FP64 form -G/36, -G/(18 1296), 1 - 1/tau, 1/(9 tau), (tau - 1/2)/36
+  double k64[kStepConstants];
+  float k32[kStepConstants];
   const double* inlet;  // inlet row velocity, u_z[Nz] then u_r[Nz] (zero until set)
   void* f[2];
   void* psi[2];
-  void* uv;         // split schedule: u_z, u_r, u^eq_z, u^eq_r, 4 planes [Nr][P] of the compute type
+  // split schedule, 4 planes [Nr][P] of the compute type: u_z, u_r, u^eq_z, u^eq_r
+  // (FP64: u_z, u_r, rho)
+  void* uv;
   // [Nr][Nz] read-back of rho, u_z, u_r for the diagnostics and the host, in the
   // compute type (FP64 for FP64 storage, else FP32: GB300's FP64 path is slow, and
   // the FP32 forms' values are FP32 numbers anyway); room for FP64 either way
@@ -42,8 +48,9 @@ struct InstDesc {
   void* ur_out;
 };
 
-// Slots of InstDesc::k64 / k32.
-enum { K_TAU, K_OMEGA, K_NEGG, K_GFAC, K_GZ, K_RHO0, K_INVRHO0, K_CMU, K_RREF, K_R0, K_RHOOUT, K_GUO };
+enum { K_TAU, K_OMEGA, K_NEGG, K_GFAC, K_GZ, K_RHO0, K_INVRHO0, K_CMU, K_RREF, K_R0, K_RHOOUT, K_GUO,
+       K_NEGG36, K_GF1296, K_OM1, K_OM9, K_CMU12 };
+static_assert(K_CMU12 + 1 == kStepConstants, "one slot per constant");
 
 // Kernel launchers (defined in amlbm_step.cu).  storage = AMLBM_STORE_*.
 // Every launcher returns the cudaGetLastError() of its launch.
@@ -62,13 +69,16 @@ cudaError_t launch_macro(int storage, int tz, int tr, const InstDesc* d_desc,
                          const int* d_tile_inst, int ntiles, int toff, int parity, cudaStream_t s);
 // Loads the code of the read-back kernel of a storage form on the current
 // device (the CUDA runtime otherwise loads it at its first launch).
-cudaError_t macro_preload(int storage);
-// Tile of the read-back kernel: 26 x 16 for the FP32-arithmetic forms (less halo
-// work per site than 32 x 8), 32 x 8 for FP64.
-inline void rb_tile(int storage, int* tz, int* tr) {
+cudaError_t macro_preload(int storage, int rz, int rr);
+// Tile of the read-back kernel of a batch whose step runs (sched, tz, tr): the step's
+// own tile on the pair schedule and for FP64 on the split one (whose force kernel
+// reads back), else 26 x 16 for the FP32-arithmetic forms (less halo work per site
+// than 32 x 8) and 32 x 8 for FP64.
+inline void rb_tile(int storage, int sched, int tz, int tr, int* rz, int* rr) {
   const bool f64 = storage == 0;  // AMLBM_STORE_F64
-  *tz = f64 ? 32 : 26;
-  *tr = f64 ? 8 : 16;
+  const bool step = sched == SCHED_PAIR || (f64 && sched == SCHED_SPLIT);
+  *rz = step ? tz : f64 ? 32 : 26;
+  *rr = step ? tr : f64 ? 8 : 16;
 }
 cudaError_t launch_init(int storage, const InstDesc* d_desc, int inst, int Nz, int Nr,
                         const double* rho, const double* uz, const double* ur, int parity,
@@ -86,9 +96,15 @@ enum InterField {
 // The timestep of instance 0 of d_desc from f[0] / psi[0] into f[1] / psi[1]
 // (FP64 / FP32 storage, no shift) together with the intermediates of the state
 // it starts from (I_COUNT planes of `plane` elements of the compute type).
-cudaError_t launch_step_inter(int storage, int tz, int tr, const InstDesc* d_desc,
-                              const int* d_tile_inst, int ntiles, void* inter, size_t plane,
-                              cudaStream_t s);
+// inter_tile() is its tile; fstar: 9 scratch planes of the FP64 form (else unused).
+cudaError_t launch_step_inter(int storage, int tz, int tr, const InstDesc* d_desc, const int* d_tile_inst,
+                              int ntiles, void* inter, size_t plane, void* fstar, cudaStream_t s);
+// FP64: 8 x 4 where 32 x 8 would leave too many SMs without a tile (pick_tile).
+inline void inter_tile(int storage, int Nz, int Nr, int* tz, int* tr) {
+  const bool small = storage == 0 && ((Nz + 31) / 32) * ((Nr + 7) / 8) < 96;  // AMLBM_STORE_F64
+  *tz = small ? 8 : 32;
+  *tr = small ? 4 : 8;
+}
 // Diagnostics (amlbm_diag.cu) of the state whose rho / u the read-back kernel
 // has written: partial sums into `partials` (nblk x 8 doubles) and the Nz column
 // radii into `cols`, then a single-block pass into out[16].
@@ -139,6 +155,18 @@ cudaError_t launch_step_pair(int storage, int tz, int tr, const InstDesc* d_desc
 // The read-back (rho, u into the read-back planes) of a pair batch, whose
 // read-back list is tiled like its step: nt tiles from toff.  And the loading of
 // that kernel's code on the current device (launches nothing).
+// The FP64 form's split schedule and read-back (amlbm_step_split64.cu): any lattice.
+// launch_step_inter64 as launch_step_inter, the collided populations going through
+// `fstar` (9 planes), which the two kernels alone use.
+int split64_tile_list(int* tz, int* tr, int cap);
+bool split64_tile_supported(int tz, int tr);
+cudaError_t launch_step_split64(int tz, int tr, const InstDesc* d_desc, const int* d_tile_inst, int ntiles,
+                                int parity, cudaStream_t s, int* ctr);
+cudaError_t launch_readback64(int tz, int tr, const InstDesc* d_desc, const int* d_tile_inst, int nt, int toff,
+                              int parity, cudaStream_t s);
+cudaError_t readback64_preload(int tz, int tr);
+cudaError_t launch_step_inter64(int tz, int tr, const InstDesc* d_desc, const int* d_tile_inst, int ntiles,
+                                double* inter, size_t plane, double* fstar, cudaStream_t s);
 cudaError_t launch_readback_pair(int storage, int tz, int tr, const InstDesc* d_desc, const int* d_tile_inst,
                                  int nt, int toff, int parity, cudaStream_t s);
 cudaError_t readback_pair_preload(int storage, int tz, int tr);
@@ -169,9 +197,10 @@ amlbm_diag_params diag_defaults(const InstDesc& d);
 std::string unstable_message(double bad);
 // Looks up, once per device and with that device current, the device address of
 // the allocation-free diagnostics' scratch array (amlbm_noalloc.cu), and loads
-// the code of the kernels that entry point launches for this storage form.
+// the code of the kernels that entry point launches for this storage form and
+// read-back tile.
 // Lattice creation calls it, so that the lookup and the loading (which the CUDA
 // runtime otherwise does lazily) happen in a call that allocates anyway.
-int noalloc_prepare(int storage);
+int noalloc_prepare(int storage, int rz, int rr);
 
 }  // namespace amlbm

@@ -80,13 +80,13 @@ int scratch_for_current_device(double** out) {
 }  // namespace
 
 namespace amlbm {
-int noalloc_prepare(int storage) {
+int noalloc_prepare(int storage, int rz, int rr) {
   double* p = nullptr;
   const int rc = scratch_for_current_device(&p);
   if (rc) return rc;
   // the code of the kernels it launches (read-back, diagnostics), so that its
   // first call loads nothing
-  if (macro_preload(storage) != cudaSuccess || diag_preload() != cudaSuccess) return AMLBM_ECUDA;
+  if (macro_preload(storage, rz, rr) != cudaSuccess || diag_preload() != cudaSuccess) return AMLBM_ECUDA;
   return AMLBM_OK;
 }
 }  // namespace amlbm

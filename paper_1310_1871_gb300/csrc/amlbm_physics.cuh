@@ -9,6 +9,8 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "amlbm.h"
 #include "amlbm_internal.cuh"
 
@@ -48,6 +50,16 @@ __device__ __forceinline__ D1 operator-(D1 a, D1 b) { return {__dsub_rn(a.v, b.v
 __device__ __forceinline__ D1 operator*(D1 a, D1 b) { return {__dmul_rn(a.v, b.v)}; }
 __device__ __forceinline__ D1 operator-(D1 a) { return {-a.v}; }
 __device__ __forceinline__ D1 fma(D1 a, D1 b, D1 c) { return {__fma_rn(a.v, b.v, c.v)}; }
+
+// FP64 runs at 1/58 of the FP32 rate on GB300 (measured: one warp instruction per
+// 16.4 clocks and SM), so an FP64 step costs what its FP64 operations cost and
+// nothing else.  The FP64 form therefore evaluates the same equations with fewer
+// of them: the stencils without their common factors (folded into the force and
+// source constants), the equilibrium, collision and sources of opposite directions
+// from one symmetric and one antisymmetric part, no arithmetic in its codec:
+// 208 operations per site against 472 in the two-kernel schedule.  The FP32
+// forms keep their own sequence of operations.
+template <class T> constexpr bool kWide = std::is_same<T, D1>::value;
 
 template <class T> struct Lane;
 template <> struct Lane<F1> { using C = float; static constexpr int N = 1; };
@@ -189,20 +201,32 @@ template <class T>
 __device__ __forceinline__ T link8(const T* p, int dz, int dr, int st) {
   return fma(lit<T>(8.0), p[dr * st + dz], -p[2 * dr * st + 2 * dz]);
 }
+// The FP64 form returns 36 times the derivative.
 template <class T>
 __device__ __forceinline__ T iso_r(const T* p, int st) {
   const T a = link8(p, 0, 1, st) - link8(p, 0, -1, st);
   const T b = (link8(p, 1, 1, st) + link8(p, -1, 1, st)) - (link8(p, 1, -1, st) + link8(p, -1, -1, st));
-  return (a + b) * lit<T>(1.0 / 36.0);
+  if constexpr (kWide<T>) return a + b;
+  else return (a + b) * lit<T>(1.0 / 36.0);
 }
 // 1D 4th-order central difference with element step `step` (Sec. II.D): the
 // inner and outer operators of d_zr psi, and the velocity gradients of the
 // sources.  (The velocity gradients do not take the isotropic stencil: its
 // diagonal taps reverse the sign of d_r u_z on a mode alternating in z, and
 // mu d_r u_z / r then amplifies that mode next to a no-slip wall.)
+// The FP64 form returns 12 times the difference.
 template <class T>
 __device__ __forceinline__ T d1(const T* p, int step) {
-  return fma(lit<T>(8.0), p[step] - p[-step], -(p[2 * step] - p[-2 * step])) * lit<T>(1.0 / 12.0);
+  const T d = fma(lit<T>(8.0), p[step] - p[-step], -(p[2 * step] - p[-2 * step]));
+  if constexpr (kWide<T>) return d;
+  else return d * lit<T>(1.0 / 12.0);
+}
+// The derivatives themselves from what iso_r, d1, sc_sums and their compositions
+// return (for the adjoint's stored intermediates).
+template <class T>
+__device__ __forceinline__ T unscale(T v, double factor) {
+  if constexpr (kWide<T>) return v * lit<T>(1.0 / factor);
+  else return v;
 }
 
 // c_i . v of direction i
@@ -272,9 +296,16 @@ __device__ __forceinline__ void guo_force(T uz, T ur, T Fz, T Fr, T* s) {
   }
   s[0] = -((s[2] + s[4]) + ((s[1] + s[3]) + ((s[5] + s[6]) + (s[7] + s[8]))));
 }
-// Shan-Chen neighbour sums sum_i W_i psi(x + c_i) c_i (Eq. scforce) around p.
+// Shan-Chen neighbour sums sum_i W_i psi(x + c_i) c_i (Eq. scforce) around p; the
+// FP64 form returns 36 times them, from the differences along the two diagonals.
 template <class T>
 __device__ __forceinline__ void sc_sums(const T* p, int Z, T& sz, T& sr) {
+  if constexpr (kWide<T>) {
+    const T u = p[Z + 1] - p[-Z - 1], w = p[-Z + 1] - p[Z - 1];
+    sz = fma(p[1] - p[-1], lit<T>(4.0), u + w);
+    sr = fma(p[Z] - p[-Z], lit<T>(4.0), u - w);
+    return;
+  }
   sz = fma(p[1] - p[-1], lit<T>(1.0 / 9.0),
            ((p[Z + 1] - p[Z - 1]) + (p[-Z + 1] - p[-Z - 1])) * lit<T>(1.0 / 36.0));
   sr = fma(p[Z] - p[-Z], lit<T>(1.0 / 9.0),
@@ -284,6 +315,12 @@ __device__ __forceinline__ void sc_sums(const T* p, int Z, T& sz, T& sr) {
 template <class T>
 struct Par {
   T tau, omega, negG, gfac, gz, rho0, inv_rho0, cmu;
+};
+// The FP64 form's constants: -G / 36, -G / (18 * 1296), 1 - 1/tau, 1/(9 tau),
+// (tau - 1/2) / 36 and -rho0, next to the ones both use.
+template <>
+struct Par<D1> {
+  D1 tau, gz, inv_rho0, rho0, negG36, gf1296, om1, om9, cmu12;
 };
 __device__ __forceinline__ float kc(const InstDesc& D, int c, float) { return D.k32[c]; }
 __device__ __forceinline__ double kc(const InstDesc& D, int c, double) { return D.k64[c]; }
@@ -297,6 +334,17 @@ __device__ __forceinline__ Par<T> par_of(const InstDesc& D) {
   using C = typename Lane<T>::C;
   Par<T> q;
   q.tau = splat<T>(kc(D, K_TAU, C()));
+  if constexpr (kWide<T>) {
+    q.gz = splat<T>(D.k64[K_GZ]);
+    q.inv_rho0 = splat<T>(D.k64[K_INVRHO0]);
+    q.rho0 = splat<T>(D.k64[K_RHO0]);
+    q.negG36 = splat<T>(D.k64[K_NEGG36]);
+    q.gf1296 = splat<T>(D.k64[K_GF1296]);
+    q.om1 = splat<T>(D.k64[K_OM1]);
+    q.om9 = splat<T>(D.k64[K_OM9]);
+    q.cmu12 = splat<T>(D.k64[K_CMU12]);
+    return q;
+  } else {
   q.omega = splat<T>(kc(D, K_OMEGA, C()));
   q.negG = splat<T>(kc(D, K_NEGG, C()));
   q.gfac = splat<T>(kc(D, K_GFAC, C()));
@@ -305,40 +353,177 @@ __device__ __forceinline__ Par<T> par_of(const InstDesc& D) {
   q.inv_rho0 = splat<T>(kc(D, K_INVRHO0, C()));
   q.cmu = splat<T>(kc(D, K_CMU, C()));
   return q;
+  }
 }
 // 1 / r of row j, r = j + r0 with r0 = r_off + 1/2 the radius of row 0 (the sum
 // is exact in either precision for the half-integer radii of the workloads)
 __device__ __forceinline__ F1 inv_r_of(F1, int j, float r0) { return rcp(F1{__int2float_rn(j) + r0}); }
 __device__ __forceinline__ D1 inv_r_of(D1, int j, double r0) { return rcp(D1{__int2double_rn(j) + r0}); }
 
+// What the site arithmetic needs of row j besides its index: 1 / r and, in the FP64
+// form, the force factors that carry the stencils' scales (formed once per row or
+// per site with the same operations).
+template <class T>
+struct Row {
+  T inv_r;
+};
+template <>
+struct Row<D1> {
+  D1 g, g9, inv36;    // of the force: -G/(18 1296) / r, 9 times that, 36 / r
+  D1 inv12, i3, ni9;  // of the sources: 12 / r, 1 / (3 r), -1 / (9 r)
+};
+template <class T>
+__device__ __forceinline__ Row<T> row_of(const Par<T>& q, int j, typename Lane<T>::C r0) {
+  Row<T> w;
+  const T inv_r = inv_r_of(T(), j, r0);
+  if constexpr (kWide<T>) {
+    w.g = q.gf1296 * inv_r;
+    w.g9 = w.g * lit<T>(9.0);
+    w.inv36 = inv_r * lit<T>(36.0);
+    w.inv12 = inv_r * lit<T>(12.0);
+    w.i3 = inv_r * lit<T>(1.0 / 3.0);
+    w.ni9 = inv_r * lit<T>(-1.0 / 9.0);
+  } else {
+    w.inv_r = inv_r;
+  }
+  return w;
+}
+
+// The force of Eq. scforce and Eq. scAxisExtra without the body force rho g_z,
+// from sc_sums, iso_r (dr0), iso_r of that (Drr) and d1 along z of d1 along r (Dzr).
+template <class T>
+__device__ __forceinline__ void forces_partial(const Par<T>& q, T psi, T sz, T sr, bool ax, T dr0, T Drr, T Dzr,
+                                               const Row<T>& w, T& Fz, T& Fr) {
+  if constexpr (kWide<T>) {
+    const T gpsi = psi * q.negG36;
+    Fz = gpsi * sz;
+    Fr = gpsi * sr;
+    if (ax) {
+      Fz = fma(psi * w.g9, Dzr, Fz);
+      Fr = fma(psi * w.g, fma(-dr0, w.inv36, Drr), Fr);
+    }
+  } else {
+    const T gpsi = psi * q.negG;
+    Fz = gpsi * sz;
+    Fr = gpsi * sr;
+    if (ax) {
+      const T g = (psi * q.gfac) * w.inv_r;
+      Fz = fma(g, Dzr, Fz);
+      Fr = fma(g, fma(-dr0, w.inv_r, Drr), Fr);
+    }
+  }
+}
 // Total force on a site (Eq. scforce, Eq. scAxisExtra, body force rho g_z).
 template <class T>
 __device__ __forceinline__ void forces(const Par<T>& q, T rho, T psi, T sz, T sr, bool ax, T dr0, T Drr,
-                                       T Dzr, T inv_r, T& Fz, T& Fr) {
-  const T gpsi = psi * q.negG;
-  Fz = gpsi * sz;
-  Fr = gpsi * sr;
-  if (ax) {
-    const T g = (psi * q.gfac) * inv_r;
-    Fz = fma(g, Dzr, Fz);
-    Fr = fma(g, fma(-dr0, inv_r, Drr), Fr);
-  }
+                                       T Dzr, const Row<T>& w, T& Fz, T& Fr) {
+  forces_partial(q, psi, sz, sr, ax, dr0, Drr, Dzr, w, Fz, Fr);
   Fz = fma(rho, q.gz, Fz);
 }
+
+// The BGK collision of a site (Eq. lbm2d): f + (f^eq - f)/tau at u^eq = v, with the
+// Guo forcing f^eq at u plus gk = 1 - 1/(2 tau) times the discrete force.  put(i, value)
+// receives the nine populations.
+//
+// FP64: with m = rho / (9 tau), the populations of a pair of opposite directions are
+// (1 - 1/tau) f + q +- k, q = W/(1/9) m (1 - 1.5 v^2 + 4.5 (c.v)^2) and k the part odd
+// in c; the Guo force adds to both parts.  The rest population is evaluated directly:
+// the FP32 forms' closure (equilibrium) guards against weights that do not sum to one,
+// an error of 1e-16 per step here.
+template <class T, class PUT>
+__device__ __forceinline__ void collide(const Par<T>& q, bool guo, T gk, const T* f, T rho, T uz, T ur, T jz, T jr,
+                                        T Fz, T Fr, T inv_rho, PUT&& put) {
+  if constexpr (kWide<T>) {
+    T vz = uz, vr = ur;
+    if (!guo) {
+      vz = fma(Fz, q.tau, jz) * inv_rho;
+      vr = fma(Fr, q.tau, jr) * inv_rho;
+    }
+    const T m9 = rho * q.om9;
+    T a9 = m9 * fma(fma(vz, vz, vr * vr), lit<T>(-1.5), lit<T>(1.0));
+    const T c9 = m9 * lit<T>(4.5), k3 = m9 * lit<T>(3.0);
+    T kz = k3 * vz, kr = k3 * vr;
+    const T sv = vz + vr, dv = vr - vz;
+    T ez = c9 * vz, er = c9 * vr, es = c9 * sv, ed = c9 * dv;
+    if (guo) {
+      const T g3 = gk * lit<T>(1.0 / 3.0);
+      a9 = fma(-g3, fma(uz, Fz, ur * Fr), a9);
+      kz = fma(g3, Fz, kz);
+      kr = fma(g3, Fr, kr);
+      ez = fma(gk, Fz, ez);
+      er = fma(gk, Fr, er);
+      es = fma(gk, Fz + Fr, es);
+      ed = fma(gk, Fr - Fz, ed);
+    }
+    const T quarter = lit<T>(0.25);
+    const T qz = fma(ez, vz, a9), qr = fma(er, vr, a9);
+    const T qs = fma(es, sv, a9), qd = fma(ed, dv, a9), ks = kz + kr, kd = kr - kz;
+    put(0, fma(q.om1, f[0], a9 * lit<T>(4.0)));
+    put(1, fma(q.om1, f[1], qz + kz));
+    put(3, fma(q.om1, f[3], qz - kz));
+    put(2, fma(q.om1, f[2], qr + kr));
+    put(4, fma(q.om1, f[4], qr - kr));
+    put(5, fma(q.om1, f[5], (qs + ks) * quarter));
+    put(7, fma(q.om1, f[7], (qs - ks) * quarter));
+    put(6, fma(q.om1, f[6], (qd + kd) * quarter));
+    put(8, fma(q.om1, f[8], (qd - kd) * quarter));
+  } else {
+    T fe[9];
+    if (guo) {
+      equilibrium(rho, uz, ur, fe);
+      T sg[9];
+      guo_force(uz, ur, Fz, Fr, sg);
+#pragma unroll
+      for (int i = 0; i < 9; ++i) put(i, fma(sg[i], gk, fma(fe[i] - f[i], q.omega, f[i])));
+    } else {
+      const T vz = fma(Fz, q.tau, jz) * inv_rho, vr = fma(Fr, q.tau, jr) * inv_rho;
+      equilibrium(rho, vz, vr, fe);
+#pragma unroll
+      for (int i = 0; i < 9; ++i) put(i, fma(fe[i] - f[i], q.omega, f[i]));
+    }
+  }
+}
+
 // Axisymmetric sources of App. A at a site: S = -rho u_r / r,
 // H_z = (mu (d_r u_z + d_z u_r) - rho u_r u_z) / r,
 // H_r = (2 mu (d_r u_r - u_r / r) - rho u_r^2) / r.
+// The FP64 form returns S / 9, H_z / 3 and H_r / 3, the terms of h_i of the axis
+// directions, from 12 times the gradients.
 template <class T>
 __device__ __forceinline__ void site_sources(const Par<T>& q, T rho, T uz, T ur, T druz, T dzur, T drur,
-                                             T inv_r, T& S_, T& Hz, T& Hr) {
-  const T mu = rho * q.cmu, rur = rho * ur;
-  S_ = -(rur * inv_r);
-  Hz = fma(mu, druz + dzur, -(rur * uz)) * inv_r;
-  Hr = fma(mu * lit<T>(2.0), fma(-ur, inv_r, drur), -(rur * ur)) * inv_r;
+                                             const Row<T>& w, T& S_, T& Hz, T& Hr) {
+  if constexpr (kWide<T>) {
+    const T mu = rho * q.cmu12, rur = rho * ur;
+    S_ = rur * w.ni9;
+    Hz = fma(mu, druz + dzur, -(rur * uz)) * w.i3;
+    Hr = fma(mu * lit<T>(2.0), fma(-ur, w.inv12, drur), -(rur * ur)) * w.i3;
+  } else {
+    const T mu = rho * q.cmu, rur = rho * ur;
+    S_ = -(rur * w.inv_r);
+    Hz = fma(mu, druz + dzur, -(rur * uz)) * w.inv_r;
+    Hr = fma(mu * lit<T>(2.0), fma(-ur, w.inv_r, drur), -(rur * ur)) * w.inv_r;
+  }
+}
+// f + h_i of one direction in the FP64 form, from what site_sources returns
+// (h_i = W_i (S + 3 c_i . H), Eq. condition_h).
+__device__ __forceinline__ D1 add_source(int i, D1 f, D1 S9, D1 Z, D1 R) {
+  const D1 quarter = lit<D1>(0.25);
+  switch (i) {
+    case 0: return fma(lit<D1>(4.0), S9, f);
+    case 1: return f + (S9 + Z);
+    case 2: return f + (S9 + R);
+    case 3: return f + (S9 - Z);
+    case 4: return f + (S9 - R);
+    case 5: return fma(quarter, S9 + (Z + R), f);
+    case 6: return fma(quarter, S9 + (R - Z), f);
+    case 7: return fma(quarter, S9 - (Z + R), f);
+    default: return fma(quarter, S9 - (R - Z), f);
+  }
 }
 // psi = rho0 (1 - exp(-rho / rho0)), Eq. psi.
 template <class T>
 __device__ __forceinline__ T psi_of(const Par<T>& q, T rho) {
+  if constexpr (kWide<T>) return fma(-q.rho0, expl(-rho * q.inv_rho0), q.rho0);
   return (lit<T>(1.0) - expl(-rho * q.inv_rho0)) * q.rho0;
 }
 
@@ -351,6 +536,11 @@ __device__ __forceinline__ void decode_values(int mode, const S* q, typename Sto
                                               typename Store<S>::C vz, typename Store<S>::C vr,
                                               typename Store<S>::C inv_rho0, typename Store<S>::C rho0,
                                               typename Store<S>::C rref, T* f) {
+  if constexpr (kWide<T>) {  // FP64 storage holds f itself
+#pragma unroll
+    for (int i = 0; i < 9; ++i) f[i] = T{q[i]};
+    return;
+  }
   const T sbt{shift_base(mode, psi, inv_rho0, rho0, rref)};
   if (mode == 3) {
     T fe[9];
@@ -389,6 +579,12 @@ __device__ __forceinline__ void encode_values(int mode, const T* fn, T rho, type
                                               uint32_t step, S* q, typename Store<S>::C& vz_out,
                                               typename Store<S>::C& vr_out) {
   using C = typename Store<S>::C;
+  if constexpr (kWide<T>) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) q[i] = fn[i].v;
+    vz_out = vr_out = C(0);
+    return;
+  }
   const C sb = shift_base(mode, psi, inv_rho0, rho0, rref);
   C fv[9], base[9];
 #pragma unroll

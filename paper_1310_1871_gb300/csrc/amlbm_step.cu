@@ -173,7 +173,7 @@ __device__ __forceinline__ void lbm_tile(const InstDesc* __restrict__ descs,
   for_tile<G::FR, G::FZ>([&](int lr, int lc) {
     const int j = j0 - G::HF + lr;
     if (j < 0 || j >= Nr) return;
-    const T inv_r = inv_r_of(T(), j, kc(D, K_R0, C()));
+    const Row<T> row = row_of(q, j, kc(D, K_R0, C()));
     const bool srow = lr >= 2 && lr < G::FR - 2;
     const T* p = sPsi + (lr + G::HP - G::HF) * G::PZ + (lc + G::HP - G::HF);
     const T psi = p[0];
@@ -197,7 +197,7 @@ __device__ __forceinline__ void lbm_tile(const InstDesc* __restrict__ descs,
       Dzr = d1(e + 2, 1);
     }
     T Fz, Fr;
-    forces(q, rho, psi, sz, sr, ax, dr0, Drr, Dzr, inv_r, Fz, Fr);
+    forces(q, rho, psi, sz, sr, ax, dr0, Drr, Dzr, row, Fz, Fr);
     const T inv_rho = rcp(rho);
     const int fi = lr * G::FZ + lc;
     const T uz = fma(Fz, lit<T>(0.5), jz) * inv_rho, ur = fma(Fr, lit<T>(0.5), jr) * inv_rho;
@@ -215,29 +215,17 @@ __device__ __forceinline__ void lbm_tile(const InstDesc* __restrict__ descs,
         o[I_FZ * iplane] = (Fz).v;
         o[I_FR * iplane] = (Fr).v;
         o[I_PSI * iplane] = (psi).v;
-        o[I_SZ * iplane] = (sz).v;
-        o[I_SR * iplane] = (sr).v;
-        o[I_DR * iplane] = (dr0).v;
-        o[I_DRR * iplane] = (Drr).v;
-        o[I_DZR * iplane] = (Dzr).v;
+        o[I_SZ * iplane] = unscale(sz, 36.0).v;
+        o[I_SR * iplane] = unscale(sr, 36.0).v;
+        o[I_DR * iplane] = unscale(dr0, 36.0).v;
+        o[I_DRR * iplane] = unscale(Drr, 1296.0).v;
+        o[I_DZR * iplane] = unscale(Dzr, 144.0).v;
       }
     }
     if ((MODE == 0 || MODE == 3) && srow && lc >= 2 && lc < G::FZ - 2) {
       T* out = sFs + (lr - 2) * G::SZ + (lc - 2);
-      T fe[9];
-      if (guo) {  // f^eq at u, plus (1 - 1/(2 tau)) times the discrete force
-        equilibrium(rho, uz, ur, fe);
-        T s[9];
-        guo_force(uz, ur, Fz, Fr, s);
-        const T gk = splat<T>(kc(D, K_GUO, C()));
-#pragma unroll
-        for (int i = 0; i < 9; ++i) out[i * G::nS] = fma(s[i], gk, fma(fe[i] - f[i], q.omega, f[i]));
-      } else {    // the velocity shift: f^eq at u^eq
-        const T vz = fma(Fz, q.tau, jz) * inv_rho, vr = fma(Fr, q.tau, jr) * inv_rho;
-        equilibrium(rho, vz, vr, fe);
-#pragma unroll
-        for (int i = 0; i < 9; ++i) out[i * G::nS] = fma(fe[i] - f[i], q.omega, f[i]);
-      }
+      collide(q, guo, splat<T>(kc(D, K_GUO, C())), f, rho, uz, ur, jz, jr, Fz, Fr, inv_rho,
+              [&](int i, T v) { out[i * G::nS] = v; });
     }
   });
   __syncthreads();
@@ -344,7 +332,7 @@ __device__ __forceinline__ void lbm_tile(const InstDesc* __restrict__ descs,
     T S_ = lit<T>(0.0), Hz = lit<T>(0.0), Hr = lit<T>(0.0);
     const bool brow = (inl && j == 0) || (outl && j == Nr - 1);  // no source on boundary rows
     if (ax && !brow) {
-      const T inv_r = inv_r_of(T(), j, kc(D, K_R0, C()));
+      const Row<T> row = row_of(q, j, kc(D, K_R0, C()));
       const int fi = (lr + 2) * G::FZ + (lc + 2);
       const T druz = d1(sUz + fi, G::FZ);
       const T dzur = d1(sUr + fi, 1);
@@ -352,20 +340,30 @@ __device__ __forceinline__ void lbm_tile(const InstDesc* __restrict__ descs,
       if constexpr (MODE == 3) {
         if (lr >= 1 && lr <= BR && lc >= 1 && lc <= BZ && k0 + lc - 1 < Nz) {
           C* o = inter + (size_t)j * P + (k0 + lc - 1);
-          o[I_G1 * iplane] = (druz).v;
-          o[I_G2 * iplane] = (dzur).v;
-          o[I_G3 * iplane] = (drur).v;
+          o[I_G1 * iplane] = unscale(druz, 12.0).v;
+          o[I_G2 * iplane] = unscale(dzur, 12.0).v;
+          o[I_G3 * iplane] = unscale(drur, 12.0).v;
         }
       }
-      site_sources(q, sRho[fi], sUz[fi], sUr[fi], druz, dzur, drur, inv_r, S_, Hz, Hr);
-      T h[9];
-      sources(S_, Hz, Hr, h);
-      if (link) {
+      site_sources(q, sRho[fi], sUz[fi], sUr[fi], druz, dzur, drur, row, S_, Hz, Hr);
+      if constexpr (kWide<T>) {
+        if (link) {
+          S_ = S_ * lit<T>(0.5);
+          Hz = Hz * lit<T>(0.5);
+          Hr = Hr * lit<T>(0.5);
+        }
 #pragma unroll
-        for (int i = 0; i < 9; ++i) sFs[i * G::nS + si] = fma(h[i], lit<T>(0.5), sFs[i * G::nS + si]);
+        for (int i = 0; i < 9; ++i) sFs[i * G::nS + si] = add_source(i, sFs[i * G::nS + si], S_, Hz, Hr);
       } else {
+        T h[9];
+        sources(S_, Hz, Hr, h);
+        if (link) {
 #pragma unroll
-        for (int i = 0; i < 9; ++i) sFs[i * G::nS + si] = sFs[i * G::nS + si] + h[i];
+          for (int i = 0; i < 9; ++i) sFs[i * G::nS + si] = fma(h[i], lit<T>(0.5), sFs[i * G::nS + si]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 9; ++i) sFs[i * G::nS + si] = sFs[i * G::nS + si] + h[i];
+        }
       }
     }
     if constexpr (MODE == 3) {
@@ -420,10 +418,15 @@ __device__ __forceinline__ void lbm_tile(const InstDesc* __restrict__ descs,
     }
     if (link && !brow) {
       const int di = (lr + 1) * G::SZ + (lc + 1);
-      T h[9];
-      sources(sS[di], sHz[di], sHr[di], h);
+      if constexpr (kWide<T>) {
 #pragma unroll
-      for (int i = 0; i < 9; ++i) fn[i] = fma(h[i], lit<T>(0.5), fn[i]);
+        for (int i = 0; i < 9; ++i) fn[i] = add_source(i, fn[i], sS[di], sHz[di], sHr[di]);
+      } else {
+        T h[9];
+        sources(sS[di], sHz[di], sHr[di], h);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) fn[i] = fma(h[i], lit<T>(0.5), fn[i]);
+      }
     }
     const T rho = moment0(fn);
     encode_site<S>(shift, fout + (size_t)j * P + k, psout + (size_t)j * P + k, plane, fn, rho,
@@ -532,7 +535,7 @@ __global__ void __launch_bounds__(NT) force_kernel(const InstDesc* __restrict__ 
   for_tile<BR, BZ>([&](int lr, int lc) {
     const int j = j0 + lr, k = k0 + lc;
     if (j >= Nr || k >= Nz) return;
-    const T inv_r = inv_r_of(T(), j, kc(D, K_R0, C()));
+    const Row<T> row = row_of(q, j, kc(D, K_R0, C()));
     const T* p = sPsi + (lr + G::HP) * G::PZ + (lc + G::HP);
     const T psi = p[0];
     T f[9];
@@ -549,7 +552,7 @@ __global__ void __launch_bounds__(NT) force_kernel(const InstDesc* __restrict__ 
       Dzr = d1(sD1 + lr * G::EZ + (lc + G::HD), 1);
     }
     T Fz, Fr;
-    forces(q, rho, psi, sz, sr, ax, dr0, Drr, Dzr, inv_r, Fz, Fr);
+    forces(q, rho, psi, sz, sr, ax, dr0, Drr, Dzr, row, Fz, Fr);
     const T inv_rho = rcp(rho);
     C* o = uv + (size_t)j * P + k;
     o[0] = (fma(Fz, lit<T>(0.5), jz) * inv_rho).v;
@@ -648,12 +651,12 @@ __global__ void __launch_bounds__(NT) stream_kernel(const InstDesc* __restrict__
     const int si = lr * G::SZ + lc;
     T S_ = lit<T>(0.0), Hz = lit<T>(0.0), Hr = lit<T>(0.0);
     if (ax) {
-      const T inv_r = inv_r_of(T(), j, kc(D, K_R0, C()));
+      const Row<T> row = row_of(q, j, kc(D, K_R0, C()));
       const int fi = (lr + 2) * G::FZ + (lc + 2);
       const T druz = d1(sUz + fi, G::FZ);
       const T dzur = d1(sUr + fi, 1);
       const T drur = d1(sUr + fi, G::FZ);
-      site_sources(q, sRho[si], sUz[fi], sUr[fi], druz, dzur, drur, inv_r, S_, Hz, Hr);
+      site_sources(q, sRho[si], sUz[fi], sUr[fi], druz, dzur, drur, row, S_, Hz, Hr);
       T h[9];
       sources(S_, Hz, Hr, h);
       if (link) {
@@ -862,8 +865,6 @@ struct TileEntry { int storage, sched, tz, tr; };
 constexpr TileEntry kTiles[] = {
     {AMLBM_STORE_F64, SCHED_FUSED, 32, 8}, {AMLBM_STORE_F64, SCHED_FUSED, 64, 8},
     {AMLBM_STORE_F64, SCHED_FUSED, 58, 8}, {AMLBM_STORE_F64, SCHED_FUSED, 26, 8},
-    {AMLBM_STORE_F64, SCHED_SPLIT, 32, 8}, {AMLBM_STORE_F64, SCHED_SPLIT, 64, 8},
-    {AMLBM_STORE_F64, SCHED_SPLIT, 32, 16},
     AMLBM_TILES_16(AMLBM_STORE_F32), AMLBM_TILES_16(AMLBM_STORE_F16), AMLBM_TILES_16(AMLBM_STORE_BF16),
 };
 #undef AMLBM_TILES_16
@@ -873,29 +874,24 @@ cudaError_t dispatch(bool macro, int sched, int tz, int tr, const InstDesc* d, c
                      int toff, int par, cudaStream_t s, int* ctr) {
   using T = typename Store<S>::T;
   if (nt <= 0) return cudaSuccess;
-  if (sched == SCHED_SPLIT && !macro) {
+  if constexpr (!std::is_same<S, double>::value) {  // the FP64 form has its own (launch_step, launch_macro)
+    if (macro) {
+      if (tz == 26 && tr == 16) return launch_t<S, T, 26, 16, 1>(d, ti, nt, toff, par, s);
+      return cudaErrorInvalidValue;
+    }
+    if (sched == SCHED_SPLIT) {
 #define AMLBM_SPLIT(TZ, TR) \
   if (tz == TZ && tr == TR) return launch_split_t<S, TZ, TR>(d, ti, nt, toff, par, s, ctr);
-    AMLBM_SPLIT(32, 8)
-    AMLBM_SPLIT(64, 8)
-    AMLBM_SPLIT(32, 16)
-    if constexpr (!std::is_same<S, double>::value) {
+      AMLBM_SPLIT(32, 8)
+      AMLBM_SPLIT(64, 8)
+      AMLBM_SPLIT(32, 16)
       AMLBM_SPLIT(64, 16)
-    }
 #undef AMLBM_SPLIT
-    return cudaErrorInvalidValue;
-  }
-#define AMLBM_TILE(TZ, TR)                                                   \
-  if (tz == TZ && tr == TR)                                                  \
-    return macro ? launch_t<S, T, TZ, TR, 1>(d, ti, nt, toff, par, s)        \
-                 : launch_t<S, T, TZ, TR, 0>(d, ti, nt, toff, par, s, nullptr, 0, ctr);
-  if (macro) {  // read-back: 32 x 8 for every storage, 26 x 16 for the FP32-arithmetic forms
-    AMLBM_TILE(32, 8)
-    if constexpr (!std::is_same<S, double>::value) {
-      AMLBM_TILE(26, 16)
+      return cudaErrorInvalidValue;
     }
-    return cudaErrorInvalidValue;
   }
+#define AMLBM_TILE(TZ, TR) \
+  if (tz == TZ && tr == TR) return launch_t<S, T, TZ, TR, 0>(d, ti, nt, toff, par, s, nullptr, 0, ctr);
   AMLBM_TILE(32, 8)
   AMLBM_TILE(64, 8)
   AMLBM_TILE(58, 8)
@@ -927,6 +923,7 @@ cudaError_t dispatch_storage(int storage, bool macro, int sched, int tz, int tr,
 
 bool tile_supported(int storage, int sched, int tz, int tr) {
   if (sched == SCHED_PAIR) return pair_tile_supported(storage, tz, tr);
+  if (sched == SCHED_SPLIT && storage == AMLBM_STORE_F64) return split64_tile_supported(tz, tr);
   for (const auto& e : kTiles)
     if (e.storage == storage && e.sched == sched && e.tz == tz && e.tr == tr) return true;
   return false;
@@ -934,6 +931,7 @@ bool tile_supported(int storage, int sched, int tz, int tr) {
 
 int tile_list(int storage, int sched, int* tz, int* tr, int cap) {
   if (sched == SCHED_PAIR) return pair_tile_list(storage, tz, tr, cap);
+  if (sched == SCHED_SPLIT && storage == AMLBM_STORE_F64) return split64_tile_list(tz, tr, cap);
   int n = 0;
   for (const auto& e : kTiles)
     if (e.storage == storage && e.sched == sched) {
@@ -949,17 +947,22 @@ cudaError_t launch_step(int storage, int sched, int tz, int tr, const InstDesc* 
     if (toff != 0) return cudaErrorInvalidValue;
     return launch_step_pair(storage, tz, tr, d, ti, nt, parity, s, ctr);
   }
+  if (sched == SCHED_SPLIT && storage == AMLBM_STORE_F64) {
+    if (toff != 0) return cudaErrorInvalidValue;
+    return launch_step_split64(tz, tr, d, ti, nt, parity, s, ctr);
+  }
   return dispatch_storage(storage, false, sched, tz, tr, d, ti, nt, toff, parity, s, ctr);
 }
 cudaError_t launch_macro(int storage, int tz, int tr, const InstDesc* d, const int* ti, int nt,
                          int toff, int parity, cudaStream_t s) {
+  if (storage == AMLBM_STORE_F64) return launch_readback64(tz, tr, d, ti, nt, toff, parity, s);
   return dispatch_storage(storage, true, SCHED_FUSED, tz, tr, d, ti, nt, toff, parity, s, nullptr);
 }
 
-cudaError_t macro_preload(int storage) {
+cudaError_t macro_preload(int storage, int rz, int rr) {
   cudaFuncAttributes a;
   switch (storage) {  // the read-back tiles of rb_tile()
-    case AMLBM_STORE_F64: return cudaFuncGetAttributes(&a, lbm_kernel<double, 32, 8, 1>);
+    case AMLBM_STORE_F64: return readback64_preload(rz, rr);
     case AMLBM_STORE_F32: return cudaFuncGetAttributes(&a, lbm_kernel<float, 26, 16, 1>);
     case AMLBM_STORE_F16: return cudaFuncGetAttributes(&a, lbm_kernel<__half, 26, 16, 1>);
     case AMLBM_STORE_BF16: return cudaFuncGetAttributes(&a, lbm_kernel<__nv_bfloat16, 26, 16, 1>);
@@ -967,13 +970,12 @@ cudaError_t macro_preload(int storage) {
   }
 }
 
-cudaError_t launch_step_inter(int storage, int tz, int tr, const InstDesc* d, const int* ti, int nt,
-                              void* inter, size_t plane, cudaStream_t s) {
-  if (storage == AMLBM_STORE_F64) {
-    if (tz == 32 && tr == 8) return launch_t<double, D1, 32, 8, 3>(d, ti, nt, 0, 0, s, inter, plane);
-  } else if (storage == AMLBM_STORE_F32) {
-    if (tz == 32 && tr == 8) return launch_t<float, F1, 32, 8, 3>(d, ti, nt, 0, 0, s, inter, plane);
-  }
+cudaError_t launch_step_inter(int storage, int tz, int tr, const InstDesc* d, const int* ti, int nt, void* inter,
+                              size_t plane, void* fstar, cudaStream_t s) {
+  if (storage == AMLBM_STORE_F64)
+    return launch_step_inter64(tz, tr, d, ti, nt, static_cast<double*>(inter), plane, static_cast<double*>(fstar), s);
+  if (storage == AMLBM_STORE_F32 && tz == 32 && tr == 8)
+    return launch_t<float, F1, 32, 8, 3>(d, ti, nt, 0, 0, s, inter, plane);
   return cudaErrorInvalidValue;
 }
 

@@ -141,7 +141,7 @@ __device__ __forceinline__ void stage_dr(const T* sPsi, T* sDr, T* sD1) {
 // lattice; psi of the two sites in ps.
 template <class T, int BZ, int BR>
 __device__ __forceinline__ void force_pair(const T* sPsi, const T* sDr, const T* sD1, const Par<T>& q, bool ax,
-                                           T inv_r, int lr, int cp, T* Fz2, T* Fr2, T* ps) {
+                                           const Row<T>& row, int lr, int cp, T* Fz2, T* Fr2, T* ps) {
   using G = PGeo<T, BZ, BR>;
   // psi rows -1..1, columns -2..3 around the pair
   T wp[3 * 6];
@@ -175,7 +175,7 @@ __device__ __forceinline__ void force_pair(const T* sPsi, const T* sDr, const T*
       for (int m = -2; m <= 2; ++m) e[m + 2] = m ? pe[m] : lit<T>(0.0);
       Dzr = d1(e + 2, 1);
     }
-    forces_partial(q, psi, sz, sr, ax, dr0, Drr, Dzr, inv_r, Fz2[s], Fr2[s]);
+    forces_partial(q, psi, sz, sr, ax, dr0, Drr, Dzr, row, Fz2[s], Fr2[s]);
   }
   ps[0] = wp[8];
   ps[1] = wp[9];
@@ -231,7 +231,7 @@ __device__ __forceinline__ void pair_tile(const InstDesc* __restrict__ descs, co
     const int j = j0 - 3 + lr;
     if (j < 0 || j >= Nr) return;
     T Fz2[2], Fr2[2], ps[2];
-    force_pair<T, BZ, BR>(sPsi, sDr, sD1, q, ax, inv_r_of(T(), j, r0c), lr, cp, Fz2, Fr2, ps);
+    force_pair<T, BZ, BR>(sPsi, sDr, sD1, q, ax, row_of(q, j, r0c), lr, cp, Fz2, Fr2, ps);
     const int fi = lr * G::FZ + 2 * cp;
     sts2(sFz + fi, Fz2[0], Fz2[1]);
     sts2(sFr + fi, Fr2[0], Fr2[1]);
@@ -274,20 +274,8 @@ __device__ __forceinline__ void pair_tile(const InstDesc* __restrict__ descs, co
       ur2[s] = ur;
       if (coll) {
         T* out = sFs + (lr - 2) * G::SZ + (2 * cp - 2) + s;
-        T fe[9];
-        if (guo) {
-          equilibrium(rho, uz, ur, fe);
-          T sg[9];
-          guo_force(uz, ur, Fz, Fr, sg);
-          const T gk = splat<T>(kc(D, K_GUO, C()));
-#pragma unroll
-          for (int i = 0; i < 9; ++i) out[i * G::nS] = fma(sg[i], gk, fma(fe[i] - f[i], q.omega, f[i]));
-        } else {
-          const T vz = fma(Fz, q.tau, jz) * inv_rho, vr = fma(Fr, q.tau, jr) * inv_rho;
-          equilibrium(rho, vz, vr, fe);
-#pragma unroll
-          for (int i = 0; i < 9; ++i) out[i * G::nS] = fma(fe[i] - f[i], q.omega, f[i]);
-        }
+        collide(q, guo, splat<T>(kc(D, K_GUO, C())), f, rho, uz, ur, jz, jr, Fz, Fr, inv_rho,
+                [&](int i, T v) { out[i * G::nS] = v; });
       }
     }
     sts2(sRho + fi, rho2[0], rho2[1]);
@@ -336,23 +324,26 @@ __device__ __forceinline__ void pair_tile(const InstDesc* __restrict__ descs, co
       wr[5] = wr0[3];
       T rr[2];
       lds2(sRho + fi, rr[0], rr[1]);
-      const T inv_r = inv_r_of(T(), j, r0c);
+      const Row<T> row = row_of(q, j, r0c);
       T* o = sFs + lr * G::SZ + 2 * cp;
-      T h[2][9];
+      T h[2][9], s3[2][3];
 #pragma unroll
       for (int s = 0; s < 2; ++s) {
         const T druz = d1(wz + 4 + s, 2);
         const T dzur = d1(wr0 + 2 + s, 1);
         const T drur = d1(wr + 4 + s, 2);
-        T S_, Hz, Hr;
-        site_sources(q, rr[s], wz[4 + s], wr[4 + s], druz, dzur, drur, inv_r, S_, Hz, Hr);
-        sources(S_, Hz, Hr, h[s]);
+        site_sources(q, rr[s], wz[4 + s], wr[4 + s], druz, dzur, drur, row, s3[s][0], s3[s][1], s3[s][2]);
+        if constexpr (!kWide<T>) sources(s3[s][0], s3[s][1], s3[s][2], h[s]);
       }
 #pragma unroll
       for (int i = 0; i < 9; ++i) {  // both sites' populations of direction i as one pair
         T a, b;
         lds2(o + i * G::nS, a, b);
-        sts2(o + i * G::nS, a + h[0][i], b + h[1][i]);
+        if constexpr (kWide<T>)
+          sts2(o + i * G::nS, add_source(i, a, s3[0][0], s3[0][1], s3[0][2]),
+               add_source(i, b, s3[1][0], s3[1][1], s3[1][2]));
+        else
+          sts2(o + i * G::nS, a + h[0][i], b + h[1][i]);
       }
     });
     __syncthreads();
@@ -480,7 +471,7 @@ __global__ void __launch_bounds__(Threads<T, BZ, BR>::value, Threads<T, BZ, BR>:
       ld2<C>(psin + 2 * plane + so, wa, wb);
     }
     T fz[2], fr[2], ps[2];
-    force_pair<T, BZ, BR>(sPsi, sDr, sD1, q, ax, inv_r_of(T(), j, r0c), lr + 3, cp + 2, fz, fr, ps);
+    force_pair<T, BZ, BR>(sPsi, sDr, sD1, q, ax, row_of(q, j, r0c), lr + 3, cp + 2, fz, fr, ps);
     C rho2[2], uz2[2], ur2[2];
 #pragma unroll
     for (int s = 0; s < 2; ++s) {

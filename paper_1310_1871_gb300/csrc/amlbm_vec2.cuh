@@ -58,21 +58,5 @@ __device__ __forceinline__ int wrap_col(int k, int Nz, bool tiny) {
   return k < 0 ? k + Nz : (k >= Nz ? k - Nz : k);
 }
 
-// The force of Eq. scforce and Eq. scAxisExtra without the body force rho g_z
-// (forces() of the fused schedule, operation for operation, up to its last
-// fused multiply-add, which the caller applies once rho is known).
-template <class T>
-__device__ __forceinline__ void forces_partial(const Par<T>& q, T psi, T sz, T sr, bool ax, T dr0, T Drr, T Dzr,
-                                               T inv_r, T& Fz, T& Fr) {
-  const T gpsi = psi * q.negG;
-  Fz = gpsi * sz;
-  Fr = gpsi * sr;
-  if (ax) {
-    const T g = (psi * q.gfac) * inv_r;
-    Fz = fma(g, Dzr, Fz);
-    Fr = fma(g, fma(-dr0, inv_r, Drr), Fr);
-  }
-}
-
 }  // namespace
 }  // namespace amlbm
