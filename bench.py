@@ -64,10 +64,10 @@ def profiled_traffic(kernel_src, kernel):
         return None
     d = json.load(open(p))
     sha = hashlib.sha256(open(kernel_src, "rb").read()).hexdigest()
-    if d.get("source_sha256") != sha:
-        return None
-    k = d.get("kernels", {}).get(kernel)
-    return k.get("dram_bytes_per_launch") if k else None
+    for part in (d, d.get("strips", {})):  # the pair schedule's tiles, and its strips
+        if part.get("source_sha256") == sha and kernel in part.get("kernels", {}):
+            return part["kernels"][kernel].get("dram_bytes_per_launch")
+    return None
 
 
 def autotune_summary(tuned):
@@ -329,8 +329,8 @@ def run_gpu(args):
                          "traffic": (round(traffic) if traffic else None),
                          "peak_kind": f"{kind} (HBM copy bandwidth)", "bytes_per_lu": BYTES_PER_LU[STORAGE],
                          "kernel": kname,
-                         "limiter": "latency of the per-tile stage chain (barrier and load stalls, 51 % issue), "
-                                    "not HBM (DRAM 12 % busy)"},
+                         "limiter": "FP32 operand bandwidth of the packed arithmetic (the FMA pipe) and the "
+                                    "warps' rounds over 1216 places, not HBM"},
             "cpu_baseline": cpu,
             "e2e": {"value": round(e2e_val, 2), "unit": UNIT, "h2d_bytes_per_step": int(h2d),
                     "d2h_bytes_per_step": int(d2h),
@@ -363,6 +363,8 @@ def kernel_name(storage, sched, tile):
     source file that holds it."""
     t = CTYPE[storage]
     csrc = os.path.join(ROOT, "paper_1310_1871_gb300", "csrc")
+    if sched == "pair" and tile[0] == 48 and storage != "f64":  # strips of tile[1] rows
+        return f"strip_step<{t}>, {tile[1]} rows", os.path.join(csrc, "amlbm_step_strip.cu")
     if sched == "pair":
         return f"pair_persistent<{t}, {tile[0]}, {tile[1]}>", os.path.join(csrc, "amlbm_step_pair.cu")
     if sched == "fused":

@@ -335,7 +335,9 @@ typedef struct amlbm_instance {
  * library's choice for every FP64 lattice, the bounded ones too, which a caller
  * cannot request it for.  PAIR:
  * the fused update with two adjacent z-sites per thread (vector loads and
- * stores, stencil taps shared by the pair); it takes periodic lattices on the
+ * stores, stencil taps shared by the pair), on tiles, or for the FP32-arithmetic
+ * forms with tile_z = 48 on strips: one warp marches over tile_r rows of 48
+ * columns (a lattice of at most 64 columns is one strip); it takes periodic lattices on the
  * axis with an even Nz, a free-slip or no-slip outer wall, the source at the
  * departure site (AMLBM_SRC_LOCAL) and either forcing, and 9 x pitch x Nr below
  * 2^31 elements.  All three give bit-identical states. */

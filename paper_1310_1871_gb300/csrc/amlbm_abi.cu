@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <functional>
 #include <new>
 #include <string>
 #include <vector>
@@ -114,6 +115,56 @@ long long count_tiles(const std::vector<amlbm_instance>& inst, int tz, int tr) {
   return n;
 }
 
+// Rows of the strips.  A warp (one strip) takes as long for a row whether its SM
+// sub-partition holds one warp or the two it has registers for (measured: 0.68 us), so a
+// step ends when 8 x 152 places that take the strips in turn are done: the H with the
+// least of that.  A strip of n rows counts a quarter of a row for each of its first 8
+// rows of psi, 0.65 for the next 4, then n + 2 whole rows, four at a time.  Measured on
+// the 64-drop sweep of 835,240 sites (us per step): H = 18 21.5 (1157 strips, one round),
+// 10 28.7, 20 24.2, 26 27.1.
+int pick_strip(const std::vector<amlbm_instance>& inst) {
+  constexpr int kPlaces = 8 * 152;
+  auto cost = [](int rows) { return 4.6 + 4.0 * ((rows + 2 + 3) / 4); };
+  int best = 2, max_rows = 0;
+  double least = 1e300;
+  for (const auto& I : inst) max_rows = std::max(max_rows, I.Nr);
+  std::vector<double> busy;
+  for (int h = 2; h <= amlbm::kStripMaxRows; h += h < 126 ? 4 : 32) {
+    long long strips = 0;
+    double sum = 0.0, longest = 0.0;
+    for (const auto& I : inst) {
+      const long long nz = amlbm::tiles_along_z(amlbm::SCHED_PAIR, amlbm::kStripWidth, I.Nz);
+      const int whole = I.Nr / h, rest = I.Nr % h;
+      strips += nz * (whole + (rest ? 1 : 0));
+      sum += nz * (whole * cost(h) + (rest ? cost(rest) : 0.0));
+      longest = std::max(longest, cost(std::min(h, I.Nr)));
+    }
+    double t = longest;
+    if (strips > 4 * kPlaces) {
+      t = sum / kPlaces + 0.5 * longest;
+    } else if (strips > kPlaces) {  // in the order of the strips
+      busy.assign(kPlaces, 0.0);
+      t = 0.0;
+      for (const auto& I : inst) {
+        const int nz = amlbm::tiles_along_z(amlbm::SCHED_PAIR, amlbm::kStripWidth, I.Nz);
+        for (int j = 0; j < I.Nr; j += h)
+          for (int z = 0; z < nz; ++z) {
+            std::pop_heap(busy.begin(), busy.end(), std::greater<double>());
+            busy.back() += cost(std::min(h, I.Nr - j));
+            t = std::max(t, busy.back());
+            std::push_heap(busy.begin(), busy.end(), std::greater<double>());
+          }
+      }
+    }
+    if (t < least) {
+      least = t;
+      best = h;
+    }
+    if (h >= max_rows) break;
+  }
+  return best;
+}
+
 // Schedule and tile when the caller gives none.
 //
 // FP64: the two kernels of amlbm_step_split64.cu, on the largest tile that still keeps
@@ -123,9 +174,9 @@ long long count_tiles(const std::vector<amlbm_instance>& inst, int tz, int tr) {
 // 1024 x 512 338 / 250 / 227 / 218 (before: 394); 330,400 sites in 25 lattices 217 / 168 /
 // 158.5 / 164.5.
 //
-// FP32 arithmetic: the pair schedule where every lattice allows it, else the fused
-// one, with the first tile of a preference list that still gives every SM two CTAs
-// over the whole batch.
+// FP32 arithmetic: the pair schedule's strips where every lattice allows it (pick_strip),
+// else the fused schedule, with the first tile of a preference list that still gives
+// every SM two CTAs over the whole batch.
 void pick_tile(int storage, const std::vector<amlbm_instance>& inst, int* sched, int* tz, int* tr) {
   if (storage == AMLBM_STORE_F64) {
     static const struct { int tz, tr, least; } pref64[] = {{32, 16, 912}, {32, 8, 96}, {16, 8, 128}, {8, 4, 0}};
@@ -136,19 +187,19 @@ void pick_tile(int storage, const std::vector<amlbm_instance>& inst, int* sched,
       if (count_tiles(inst, t.tz, t.tr) >= t.least) return;
     }
   }
+  if (all_pair_ok(inst)) {
+    *sched = amlbm::SCHED_PAIR;
+    *tz = amlbm::kStripWidth;
+    *tr = pick_strip(inst);
+    return;
+  }
   static const int pref32[][2] = {{26, 16}, {64, 8}, {32, 8}};
-  static const int prefpair[][2] = {{64, 24}, {40, 24}, {24, 16}};
-  const bool pair = all_pair_ok(inst);
-  const int(*pref)[2] = pair ? prefpair : pref32;
-  *sched = pair ? amlbm::SCHED_PAIR : amlbm::SCHED_FUSED;
-  for (int c = 0; c < 3; ++c) {
-    *tz = pref[c][0];
-    *tr = pref[c][1];
+  *sched = amlbm::SCHED_FUSED;
+  for (const auto& t : pref32) {
+    *tz = t[0];
+    *tr = t[1];
     if (count_tiles(inst, *tz, *tr) >= 2 * 152) return;
   }
-  *sched = amlbm::SCHED_FUSED;
-  *tz = 32;
-  *tr = 8;
 }
 
 // Shift code the kernels use: 0 none, 1 global rho_ref, 2 local (from psi),
@@ -223,7 +274,7 @@ Layout make_layout(const std::vector<amlbm_instance>& inst, int storage, int tz,
   auto take = [&](size_t bytes) { const size_t at = o; o = align_up(o + bytes); return at; };
   const size_t n = inst.size();
   for (const auto& I : inst) {
-    L.ntiles += ((I.Nz + tz - 1) / tz) * ((I.Nr + tr - 1) / tr);
+    L.ntiles += amlbm::tiles_along_z(sched, tz, I.Nz) * ((I.Nr + tr - 1) / tr);
     int rz, rr;
     amlbm::rb_tile(storage, sched, tz, tr, &rz, &rr);
     L.rb_ntiles += ((I.Nz + rz - 1) / rz) * ((I.Nr + rr - 1) / rr);
@@ -271,6 +322,7 @@ struct amlbm_batch {
   char* arena = nullptr;
   size_t arena_bytes = 0;
   bool owns = false;
+  int form = -1;  // launch_step_strip
   Layout L;
   std::vector<InstDesc> desc;
   std::vector<long long> steps;  // per instance, since its fields were set
@@ -295,7 +347,7 @@ namespace {
 
 int launch_steps_direct(amlbm_batch* b, int n) {
   for (int s = 0; s < n; ++s) {
-    const cudaError_t e = amlbm::launch_step(b->storage, b->sched, b->tz, b->tr, b->d_desc, b->d_tiles,
+    const cudaError_t e = amlbm::launch_step(b->storage, b->sched, b->form, b->tz, b->tr, b->d_desc, b->d_tiles,
                                              b->L.ntiles, 0, b->parity, b->stream, b->d_ctr);
     if (e != cudaSuccess) return fail(AMLBM_ECUDA, std::string("step kernel: ") + cudaGetErrorString(e));
     b->parity ^= 1;
@@ -310,7 +362,7 @@ int ensure_graph(amlbm_batch* b, int parity) {
   int p = parity;
   cudaError_t e = cudaSuccess;
   for (int s = 0; s < b->graph_chunk && e == cudaSuccess; ++s) {
-    e = amlbm::launch_step(b->storage, b->sched, b->tz, b->tr, b->d_desc, b->d_tiles, b->L.ntiles, 0, p,
+    e = amlbm::launch_step(b->storage, b->sched, b->form, b->tz, b->tr, b->d_desc, b->d_tiles, b->L.ntiles, 0, p,
                            b->stream, b->d_ctr);
     p ^= 1;
   }
@@ -412,6 +464,7 @@ int batch_build(const std::vector<amlbm_instance>& inst, const amlbm_tune* tune,
     d.zbc = I.bc.z_bc;
     d.rlo = I.bc.r_lo;
     d.forcing = I.bc.forcing;
+    const bool plain = d.axisym && d.forcing == AMLBM_FORCE_SHIFT;
     // 1 = stochastic rounding of the 16-bit stores.  Default: stochastic for BF16
     // with the W_i s shifts (measured: an order of magnitude more accurate there),
     // to nearest for FP16 and for the equilibrium shift (no gain measured)
@@ -419,7 +472,9 @@ int batch_build(const std::vector<amlbm_instance>& inst, const amlbm_tune* tune,
     d.rounding = (storage != AMLBM_STORE_F16 && storage != AMLBM_STORE_BF16) ? 0
                : I.bc.rounding == AMLBM_ROUND_STOCHASTIC ? 1
                : I.bc.rounding == AMLBM_ROUND_NEAREST ? 0 : (sr_default ? 1 : 0);
-    d.tiles_z = (I.Nz + tz - 1) / tz;
+    const int form = plain && d.rounding == (sr_default ? 1 : 0) ? d.shift : -1;
+    b->form = i == 0 || form == b->form ? form : -1;
+    d.tiles_z = amlbm::tiles_along_z(sched, tz, I.Nz);
     d.tiles_r = (I.Nr + tr - 1) / tr;
     d.tile_base = (int)tiles.size();
     int rz, rr;
@@ -497,7 +552,7 @@ int batch_build(const std::vector<amlbm_instance>& inst, const amlbm_tune* tune,
   amlbm::noalloc_prepare(storage, rz, rr);
   // the pair read-back's code, loaded now for the same reason (its first use
   // may be an allocation-free diagnostics call)
-  if (sched == amlbm::SCHED_PAIR) amlbm::readback_pair_preload(storage, tz, tr);
+  if (sched == amlbm::SCHED_PAIR) amlbm::readback_pair_preload(storage, rz, rr);
   *out = b;
   return AMLBM_OK;
 }
@@ -556,11 +611,10 @@ int set_inlet(amlbm_batch* b, int k, const double* uz, const double* ur) {
 
 // rho and u of nt tiles of the read-back list from toff into the read-back planes
 cudaError_t launch_readback(amlbm_batch* b, int nt, int toff) {
-  if (b->sched == amlbm::SCHED_PAIR)
-    return amlbm::launch_readback_pair(b->storage, b->tz, b->tr, b->d_desc, b->d_rb_tiles, nt, toff, b->parity,
-                                       b->stream);
   int rz, rr;
   amlbm::rb_tile(b->storage, b->sched, b->tz, b->tr, &rz, &rr);
+  if (b->sched == amlbm::SCHED_PAIR)
+    return amlbm::launch_readback_pair(b->storage, rz, rr, b->d_desc, b->d_rb_tiles, nt, toff, b->parity, b->stream);
   return amlbm::launch_macro(b->storage, rz, rr, b->d_desc, b->d_rb_tiles, nt, toff, b->parity, b->stream);
 }
 
@@ -760,7 +814,7 @@ int diag_host(amlbm_batch* b, int k, const amlbm_diag_params* dp, amlbm_diag* ou
 extern "C" {
 
 const char* amlbm_last_error(void) { return g_err.c_str(); }
-const char* amlbm_version(void) { return "amlbm 0.2 (sm_103a)"; }
+const char* amlbm_version(void) { return "amlbm 0.3 (sm_103a)"; }
 
 int amlbm_tiles(int storage, int schedule, int* tz, int* tr, int cap) {
   return amlbm::tile_list(storage, schedule, tz, tr, cap);

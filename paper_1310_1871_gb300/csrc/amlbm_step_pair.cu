@@ -558,8 +558,11 @@ cudaError_t launch_readback_t(const InstDesc* d, const int* ti, int nt, int toff
 }
 
 struct PairTile { int storage, tz, tr; };
-#define AMLBM_PAIR_TILES(ST) {ST, 40, 24}, {ST, 48, 20}, {ST, 64, 24}, {ST, 32, 16}, {ST, 48, 16}, \
-                             {ST, 24, 16}, {ST, 64, 16}, {ST, 32, 32}
+#define AMLBM_PAIR_TILES(ST) {ST, 40, 24}, {ST, 64, 24}, {ST, 32, 16}, {ST, 24, 16}, {ST, 64, 16}, {ST, 32, 32}, \
+    {ST, kStripWidth, 2}, {ST, kStripWidth, 6}, {ST, kStripWidth, 10}, {ST, kStripWidth, 14},                \
+    {ST, kStripWidth, 16}, {ST, kStripWidth, 18}, {ST, kStripWidth, 20}, {ST, kStripWidth, 26},              \
+    {ST, kStripWidth, 34}, {ST, kStripWidth, 46}, {ST, kStripWidth, 66}, {ST, kStripWidth, 94},              \
+    {ST, kStripWidth, 126}, {ST, kStripWidth, 198}
 constexpr PairTile kPairTiles[] = {
     {AMLBM_STORE_F64, 32, 8}, {AMLBM_STORE_F64, 28, 8},
     AMLBM_PAIR_TILES(AMLBM_STORE_F32), AMLBM_PAIR_TILES(AMLBM_STORE_F16), AMLBM_PAIR_TILES(AMLBM_STORE_BF16),
@@ -585,10 +588,8 @@ cudaError_t pair_dispatch(int kind, int tz, int tr, const InstDesc* d, const int
     AMLBM_PT(28, 8)
   } else {
     AMLBM_PT(40, 24)
-    AMLBM_PT(48, 20)
     AMLBM_PT(64, 24)
     AMLBM_PT(32, 16)
-    AMLBM_PT(48, 16)
     AMLBM_PT(24, 16)
     AMLBM_PT(64, 16)
     AMLBM_PT(32, 32)
@@ -600,6 +601,7 @@ cudaError_t pair_dispatch(int kind, int tz, int tr, const InstDesc* d, const int
 }  // namespace
 
 bool pair_tile_supported(int storage, int tz, int tr) {
+  if (storage != AMLBM_STORE_F64 && tz == kStripWidth && strip_rows_ok(tr)) return true;
   for (const auto& e : kPairTiles)
     if (e.storage == storage && e.tz == tz && e.tr == tr) return true;
   return false;
@@ -626,8 +628,9 @@ static cudaError_t pair_kind(int kind, int storage, int tz, int tr, const InstDe
   }
 }
 
-cudaError_t launch_step_pair(int storage, int tz, int tr, const InstDesc* d, const int* ti, int nt, int parity,
+cudaError_t launch_step_pair(int storage, int form, int tz, int tr, const InstDesc* d, const int* ti, int nt, int parity,
                              cudaStream_t s, int* ctr) {
+  if (storage != AMLBM_STORE_F64 && tz == kStripWidth) return launch_step_strip(storage, form, tr, d, ti, nt, parity, s, ctr);
   return pair_kind(0, storage, tz, tr, d, ti, nt, 0, parity, s, ctr);
 }
 
