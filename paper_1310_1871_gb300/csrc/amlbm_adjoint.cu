@@ -4,21 +4,35 @@
 // checkpointed driver behind amlbm_adjoint / amlbm_objective.
 //
 // The forward intermediates of every state of a checkpoint segment are written
-// while the segment is recomputed (lbm_kernel MODE 3: the step and the
-// intermediates of the state it starts from in one pass).  One adjoint step
-// (lambda^{n+1} -> lambda^n, state f^n) then runs as:
-//   post   : mu = transpose of the streaming map (a gather), then the adjoint of
-//            the BGK collision and of the sources S, H_z, H_r  -> rho, u, u^eq,
-//            velocity-gradient adjoints, tau part
-//   vel    : transposed gradient stencils with the u ghosts folded back, the
-//            adjoint of u = (j + F/2)/rho and u^eq = (j + tau F)/rho, and at the
-//            same site the adjoint of F_SC (Eq. scforce) and F^gamma (Eq.
-//            scAxisExtra) (local psi factor, d_zr, d_rr, d_r parts), G part
-//   deriv  : transposed 1D d_z (of d_zr) and isotropic d_r (of d_rr)
-//   final  : transposed Shan-Chen neighbour sum, 1D d_r and isotropic d_r on psi,
-//            psi ghosts folded onto their mirrors, d psi/d rho, and
-//            lambda^n_i = (1 - omega) mu_i + rho_bar + c_i . j_bar.
-// All kernels are gathers (no atomics), so the sweep is deterministic.
+// while the segment is recomputed (launch_step_inter: the step and the
+// intermediates of the state it starts from).  One adjoint step (lambda^{n+1} ->
+// lambda^n, state f^n) then runs as two kernels:
+//   adj_local : mu = transpose of the streaming map (a gather); the adjoints of the
+//               sources' velocity gradients on the tile and two sites around it; then
+//               per site the adjoint of the BGK collision and of the sources S, H_z,
+//               H_r, the transposed gradient stencils, the adjoint of
+//               u = (j + F/2)/rho and u^eq = (j + tau F)/rho, of F_SC (Eq. scforce) and
+//               F^gamma (Eq. scAxisExtra); G and tau parts
+//   adj_psi   : transposed 1D d_z (of d_zr) and isotropic d_r (of d_rr) on the tile and
+//               two sites around it; then the transposed Shan-Chen neighbour sum, 1D d_r
+//               and isotropic d_r on psi, d psi/d rho, and
+//               lambda^n_i = (1 - omega) mu_i + rho_bar + c_i . j_bar
+// (four kernels and 30 planes of intermediates before: the small lattices of these
+// runs are bound by the chain of launches and memory round trips, FP64 by its
+// operations).  Ghost rows: a field mirrored with sign s about a boundary and read by
+// a stencil that is antisymmetric (symmetric) in r has as transpose the stencil's own
+// transpose on the adjoint field mirrored with sign -s (s), so the folds of the ghost rows
+// need no terms of their own.  All kernels are gathers (no atomics): the sweep is
+// deterministic.
+//
+// Collision: with the moments M0 = sum W mu, M = sum W c mu, MM = sum W c c mu of the
+// gathered mu, the adjoint of f^eq is a quadratic form in u^eq: 57 operations instead of
+// nine separate terms (about 190).
+//
+// Measured (GB300, ncu, one backward step, cold caches; the four kernels before): FP32,
+// 512 x 128: 21 us (45); FP64, 256 x 128: 36 us (68), 271 FP64 operations per site (543).
+// A gradient of the differentiable drop, 512 x 128, T = 100, checkpoints every 10, FP32:
+// 2.8 ms (5.2); 256 x 128, T = 50, FP64: 4.0 ms (5.6).
 
 #include <cuda_runtime.h>
 
@@ -30,6 +44,7 @@
 
 #include "amlbm.h"
 #include "amlbm_internal.cuh"
+#include "amlbm_launch.cuh"
 
 namespace amlbm {
 namespace {
@@ -52,42 +67,28 @@ __host__ __device__ constexpr int aopp(int i) {
 }
 
 // Periodic wrap of a column that lies a few sites outside [0, Nz) (no
-// division: stencil offsets are at most 4, so one or two corrections suffice
-// unless Nz is smaller than that).
+// division: stencil offsets are at most 4 beyond a tile, so one or two corrections
+// suffice unless Nz is smaller than that).
 __device__ __forceinline__ int wz(int k, int Nz) {
   while (k < 0) k += Nz;
   while (k >= Nz) k -= Nz;
   return k;
 }
+// The lattice row that a row up to Nr ghosts beyond the axis or the wall mirrors.
+__device__ __forceinline__ int mirror_row(int j, int Nr) { return j < 0 ? -1 - j : j >= Nr ? 2 * Nr - 1 - j : j; }
 
 template <class C>
 struct Adj {
   int Nz, Nr, P, wall, axisym;
   size_t plane;
-  C tau, omega, G, rho0, gz, inv_rho0;
+  C tau, omega, G, gz, inv_rho0;
   const C* lam_in;
   C* lam_out;
   const C* f;      // state f^n, 9 planes
   const C* inter;  // I_COUNT planes
-  C* mu;           // 9 planes
-  C *rhob, *uzb, *urb, *vzb, *vrb, *g1b, *g2b, *g3b, *jzb, *jrb, *Fzb, *Frb;
-  C *psib, *qz, *qr, *dzrb, *drrb, *drdb, *eb;
-  C* drpb;  // d_r psi adjoint on rows -2 .. Nr+1 (row offset 2)
+  C *rhob, *jzb, *jrb, *psib, *qz, *qr, *dzrb, *drrb, *drdb;  // adjoints, [Nr][P] each
   double *accG, *accT;
 };
-
-// value of a [Nr][P] field at (k, j), zero outside the real rows
-template <class C>
-__device__ __forceinline__ C at(const C* a, int k, int j, const Adj<C>& A) {
-  if (j < 0 || j >= A.Nr) return C(0);
-  return a[(size_t)j * A.P + wz(k, A.Nz)];
-}
-// d_r psi adjoint on the padded rows -2 .. Nr+1, zero outside
-template <class C>
-__device__ __forceinline__ C atpad(const C* a, int k, int j, const Adj<C>& A) {
-  if (j < -2 || j > A.Nr + 1) return C(0);
-  return a[(size_t)(j + 2) * A.P + wz(k, A.Nz)];
-}
 
 template <class C>
 __device__ __forceinline__ C feq_std(int i, C rho, C vz, C vr) {
@@ -95,332 +96,303 @@ __device__ __forceinline__ C feq_std(int i, C rho, C vz, C vr) {
   return C(aw(i)) * rho * (C(1) + C(3) * cv + C(4.5) * cv * cv - C(1.5) * (vz * vz + vr * vr));
 }
 
-// ---- shared-memory windows of the tiled transposed kernels
-// A block of ATZ x ATR threads handles the ATZ x ATR sites (k0 + tx, j0 + ty).  A
-// window holds a [Nr][P] field on rows j0 - HR .. j0 + ATR - 1 + HR and columns
-// k0 - 2 .. k0 + ATZ + 1 (wrapped in z), with the value the global accessors give
-// outside the stored rows (zero), so the transposed stencils read it exactly as
-// they would read global memory.  Blocks away from the axis and the wall load only
-// the rows their own sites' stencils reach (radius 2).
-constexpr int ATZ = 32, ATR = 8, ANT = ATZ * ATR;
-
-template <class C, int HR>
-struct Win {
-  static constexpr int W = ATZ + 4, H = ATR + 2 * HR;
-  C v[H * W];
-};
-
-template <bool PAD, class C, int HR>
-__device__ __forceinline__ void load_win(Win<C, HR>& w, const C* g, int k0, int j0, bool near_edge,
-                                         const Adj<C>& A) {
-  constexpr int W = Win<C, HR>::W;
-  const int r_lo = near_edge ? 0 : HR - 2, r_hi = near_edge ? Win<C, HR>::H : HR + ATR + 2;
-  for (int i = r_lo * W + threadIdx.x; i < r_hi * W; i += ANT) {
-    const int rr = i / W, cc = i - rr * W;
-    const int y = j0 - HR + rr, k = k0 - 2 + cc;
-    w.v[i] = PAD ? atpad(g, k, y, A) : at(g, k, y, A);
+// mu_q at the lattice site (k, j): lambda where population q leaving it arrives
+// (Sec. II.E maps).
+template <class C>
+__device__ __forceinline__ C arrived(const Adj<C>& A, int q, int k, int j) {
+  int yk = k, yj = j + acr(q), d = q;
+  if (yj < 0) {
+    yj = 0; d = amirror(q);
+  } else if (yj >= A.Nr) {
+    yj = A.Nr - 1;
+    d = A.wall == AMLBM_WALL_NOSLIP ? aopp(q) : amirror(q);
   }
+  if (acz(q) != 0 && !(d == aopp(q) && yj == j)) {
+    yk += acz(q);
+    yk = yk < 0 ? A.Nz - 1 : yk == A.Nz ? 0 : yk;
+  }
+  return A.lam_in[d * A.plane + (size_t)yj * A.P + yk];
 }
-
-template <class C, int HR>
-__device__ __forceinline__ C wat(const Win<C, HR>& w, int k, int y, int k0, int j0) {
-  return w.v[(y - j0 + HR) * Win<C, HR>::W + (k - k0 + 2)];
+// 9 sum W c_z mu and 9 sum W c_r mu from mu of the eight moving populations.
+template <class C>
+__device__ __forceinline__ C first_z(const C* mu) {
+  return (mu[1] - mu[3]) + C(0.25) * ((mu[5] - mu[7]) + (mu[8] - mu[6]));
 }
-
-// Transpose of the isotropic derivative along r (AX = 1) or z (AX = 0) at the
-// (possibly ghost) position (k, j), on a window:
-//   sum_i c_i,AX (8 g(y - c_i) - g(y - 2 c_i)) / 36.
-template <int AX, class C, int HR>
-__device__ __forceinline__ C iso_tw(const Win<C, HR>& g, int k, int j, int k0, int j0) {
+template <class C>
+__device__ __forceinline__ C first_r(const C* mu) {
+  return (mu[2] - mu[4]) + C(0.25) * ((mu[5] - mu[7]) + (mu[6] - mu[8]));
+}
+// Transposes of the stencils at p, rows st apart (isotropic d_r: 36 times it; 1D
+// difference with element step e: 12 times it).
+template <class C>
+__device__ __forceinline__ C iso_t(const C* p, int st) {
   C s = C(0);
 #pragma unroll
-  for (int i = 1; i < 9; ++i) {
-    const int c = AX ? acr(i) : acz(i);
-    if (c == 0) continue;
-    const C a = wat(g, k - acz(i), j - acr(i), k0, j0);
-    const C b = wat(g, k - 2 * acz(i), j - 2 * acr(i), k0, j0);
-    s += C(c) * (C(8) * a - b);
-  }
-  return s * C(1.0 / 36.0);
+  for (int dz = -1; dz <= 1; ++dz)
+    s += C(8) * (p[-st + dz] - p[st + dz]) - (p[2 * (-st + dz)] - p[2 * (st + dz)]);
+  return s;
 }
-
-// Transpose of the 1D 4th-order difference along r (AX = 1) or z (AX = 0) at the
-// (possibly ghost) position (k, j), on a window.  The forward operator
-// (8 (g(y + e) - g(y - e)) - (g(y + 2e) - g(y - 2e))) / 12 is antisymmetric, so
-// its transpose is its negative.
-template <int AX, class C, int HR>
-__device__ __forceinline__ C d1_tw(const Win<C, HR>& g, int k, int j, int k0, int j0) {
-  const int ez = AX ? 0 : 1, er = AX ? 1 : 0;
-  const C a = wat(g, k + ez, j + er, k0, j0) - wat(g, k - ez, j - er, k0, j0);
-  const C b = wat(g, k + 2 * ez, j + 2 * er, k0, j0) - wat(g, k - 2 * ez, j - 2 * er, k0, j0);
-  return -(C(8) * a - b) * C(1.0 / 12.0);
-}
-
-// ---- post: inverse streaming, collision and source adjoints (per real site)
 template <class C>
-__global__ void __launch_bounds__(ANT) adj_post(Adj<C> A) {
-  // lambda^{n+1} on the tile + 1 (9 planes), the rows and columns every arrival
-  // site of the tile's populations lies in
-  constexpr int W = ATZ + 2, H = ATR + 2;
-  __shared__ C wl[9][H * W];
-  const int k0 = blockIdx.x * ATZ, j0 = blockIdx.y * ATR;
-  for (int i = threadIdx.x; i < H * W; i += ANT) {
-    const int rr = i / W, cc = i - rr * W;
-    const int y = j0 - 1 + rr, x = k0 - 1 + cc;
-    const bool in = y >= 0 && y < A.Nr;
-    const size_t g = in ? (size_t)y * A.P + wz(x, A.Nz) : 0;
-#pragma unroll
-    for (int d = 0; d < 9; ++d) wl[d][i] = in ? A.lam_in[d * A.plane + g] : C(0);
+__device__ __forceinline__ C d1_t(const C* p, int e) {
+  return C(8) * (p[-e] - p[e]) - (p[-2 * e] - p[2 * e]);
+}
+
+// Tiles of ATZ x BR sites, one thread per site.
+constexpr int ATZ = 32;
+template <int NT, int ROWS, int W, class F>
+__device__ __forceinline__ void for_region(F&& body) {
+  for (int t = threadIdx.x; t < ROWS * W; t += NT) {
+    const int lr = t / W;
+    body(lr, t - lr * W);
   }
+}
+
+template <class C, int BR>
+__global__ void __launch_bounds__(ATZ * BR) adj_local(Adj<C> A) {
+  constexpr int NT = ATZ * BR, W = ATZ + 4;
+  __shared__ C g1[(BR + 4) * W];    // adjoint of d_r u_z (and of d_z u_r): the tile + 2, but the corners
+  __shared__ C g3[(BR + 4) * ATZ];  // adjoint of d_r u_r: rows + 2
+  __shared__ C s_ir[BR + 4];        // 1 / r of rows j0 - 2 ..
+  const int k0 = blockIdx.x * ATZ, j0 = blockIdx.y * BR;
+  const int tx = (int)threadIdx.x % ATZ, ty = (int)threadIdx.x / ATZ, k = k0 + tx, j = j0 + ty;
+  const bool in = k < A.Nz && j < A.Nr;
+  const C cmu = (A.tau - C(0.5)) * C(1.0 / 3.0);
+  const size_t o = (size_t)(in ? j : 0) * A.P + (in ? k : 0);
+  if (threadIdx.x < BR + 4) s_ir[threadIdx.x] = C(1) / (C(mirror_row(j0 - 2 + (int)threadIdx.x, A.Nr)) + C(0.5));
   __syncthreads();
-  const int k = k0 + (int)threadIdx.x % ATZ, j = j0 + (int)threadIdx.x / ATZ;
-  if (k >= A.Nz || j >= A.Nr) return;
-  const size_t o = (size_t)j * A.P + k;
-  const bool noslip = A.wall == AMLBM_WALL_NOSLIP;
+  pdl_wait();
   C mu[9];
+  if (in) {
 #pragma unroll
-  for (int q = 0; q < 9; ++q) {
-    // where population q leaving (k, j) arrives after streaming (Sec. II.E maps)
-    int yk = k + acz(q), yj = j + acr(q), d = q;
-    if (yj < 0) {
-      yj = 0; d = amirror(q);
-    } else if (yj >= A.Nr) {
-      if (noslip) { yk = k; yj = A.Nr - 1; d = aopp(q); }
-      else { yj = A.Nr - 1; d = amirror(q); }
-    }
-    mu[q] = wl[d][(yj - j0 + 1) * W + (yk - k0 + 1)];
-    A.mu[q * A.plane + o] = mu[q];
+    for (int q = 0; q < 9; ++q) mu[q] = arrived(A, q, k, j);
   }
+  if (A.axisym) {
+    const C wall_z = A.wall == AMLBM_WALL_NOSLIP ? C(1) : C(-1);  // minus the sign u_z is mirrored with
+    // g_1 = g_2 = Hz_bar mu / r, g_3 = 2 Hr_bar mu / r with H_bar = 3 sum W c mu_q
+    for_region<NT, BR + 4, ATZ>([&](int lr, int lc) {
+      const int y = j0 - 2 + lr, x = k0 + lc;
+      if (y > A.Nr + 1 || x >= A.Nz) return;
+      const int m = mirror_row(y, A.Nr);
+      C v[9];
+#pragma unroll
+      for (int q = 1; q < 9; ++q) v[q] = arrived(A, q, x, m);
+      const C c = A.inter[I_RHO * A.plane + (size_t)m * A.P + x] * (cmu * s_ir[lr]) * C(1.0 / 3.0);
+      const C sz = y < 0 ? C(-1) : y >= A.Nr ? wall_z : C(1);
+      g1[lr * W + lc + 2] = sz * c * first_z(v);
+      g3[lr * ATZ + lc] = C(2) * c * first_r(v);
+    });
+    for_region<NT, BR, 4>([&](int lr, int lc) {  // two columns on either side
+      const int y = j0 + lr;
+      if (y >= A.Nr) return;
+      const int c0 = lc < 2 ? lc : ATZ + lc, x = wz(k0 - 2 + c0, A.Nz);
+      C v[9];
+#pragma unroll
+      for (int q = 1; q < 9; ++q)
+        if (acz(q) != 0) v[q] = arrived(A, q, x, y);
+      g1[(lr + 2) * W + c0] = A.inter[I_RHO * A.plane + (size_t)y * A.P + x] * (cmu * s_ir[lr + 2]) * C(1.0 / 3.0) *
+                              first_z(v);
+    });
+    // a ragged tile: its last columns' right-hand neighbours wrap inside the tile
+    if (k0 + ATZ > A.Nz) {
+      for_region<NT, BR, 2>([&](int lr, int lc) {
+        const int y = j0 + lr, c0 = A.Nz - k0 + lc;
+        if (y >= A.Nr || c0 >= ATZ + 2) return;
+        const int x = wz(A.Nz + lc, A.Nz);
+        C v[9];
+#pragma unroll
+        for (int q = 1; q < 9; ++q)
+          if (acz(q) != 0) v[q] = arrived(A, q, x, y);
+        g1[(lr + 2) * W + c0 + 2] = A.inter[I_RHO * A.plane + (size_t)y * A.P + x] * (cmu * s_ir[lr + 2]) *
+                                    C(1.0 / 3.0) * first_z(v);
+      });
+    }
+    __syncthreads();
+  }
+  if (!in) return;
   const C* I = A.inter + o;
   const C rho = I[I_RHO * A.plane], vz = I[I_VZ * A.plane], vr = I[I_VR * A.plane];
   const C uz = I[I_UZ * A.plane], ur = I[I_UR * A.plane];
-  C rb = C(0), vzb = C(0), vrb = C(0), tb = C(0);
-  const C irho = C(1) / rho;
+  // moments of mu, 9 times: M0, M_z, M_r, M_zz, M_zr, M_rr
+  const C pz = mu[1] + mu[3], pr = mu[2] + mu[4], ps = mu[5] + mu[7], pd = mu[6] + mu[8];
+  const C diag = C(0.25) * (ps + pd);
+  const C Mzz = pz + diag, Mrr = pr + diag, Mzr = C(0.25) * (ps - pd);
+  const C M0 = C(4) * mu[0] + (pz + pr) + diag;
+  const C Mz = first_z(mu), Mr = first_r(mu);
+  const C tz = vz * Mzz + vr * Mzr, tr = vz * Mzr + vr * Mrr;
+  const C Aq = C(1) - C(1.5) * (vz * vz + vr * vr);
+  // sum mu f^eq / rho, and the adjoints of u^eq
+  const C fe = C(1.0 / 9.0) * (Aq * M0 + C(4.5) * (vz * tz + vr * tr) + C(3) * (vz * Mz + vr * Mr));
+  // tau part, -omega^2 sum mu (f^eq - f).  In FP32 term by term: mu is nearly the same
+  // for all directions, so the sums of mu f^eq and mu f agree to almost every bit, and
+  // their difference would keep only rounding.
+  C tb = C(0);
+  if constexpr (sizeof(C) == 8) {
 #pragma unroll
-  for (int q = 0; q < 9; ++q) {
-    const C fe = feq_std(q, rho, vz, vr);
-    const C cv = C(acz(q)) * vz + C(acr(q)) * vr;
-    const C m = A.omega * mu[q];
-    rb += m * fe * irho;
-    const C com = m * C(aw(q)) * rho;
-    vzb += com * (C(3) * C(acz(q)) + C(9) * cv * C(acz(q)) - C(3) * vz);
-    vrb += com * (C(3) * C(acr(q)) + C(9) * cv * C(acr(q)) - C(3) * vr);
-    tb += -A.omega * A.omega * mu[q] * (fe - A.f[q * A.plane + o]);
+    for (int q = 0; q < 9; ++q) tb += mu[q] * A.f[q * A.plane + o];
+    tb -= rho * fe;
+  } else {
+#pragma unroll
+    for (int q = 0; q < 9; ++q) tb += mu[q] * (A.f[q * A.plane + o] - feq_std(q, rho, vz, vr));
   }
-  C uzb = C(0), urb = C(0), g1b = C(0), g2b = C(0), g3b = C(0);
+  tb *= A.omega * A.omega;
+  C rb = A.omega * fe;
+  const C com = A.omega * rho * C(1.0 / 3.0);
+  const C vzb = com * (Mz + C(3) * tz - vz * M0), vrb = com * (Mr + C(3) * tr - vr * M0);
+  C uzb = C(0), urb = C(0);
+  const C irr = A.axisym ? s_ir[ty + 2] : C(0);
   if (A.axisym) {
-    C Sb = C(0), Hzb = C(0), Hrb = C(0);
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-      Sb += mu[q] * C(aw(q));
-      Hzb += C(3) * mu[q] * C(aw(q)) * C(acz(q));
-      Hrb += C(3) * mu[q] * C(aw(q)) * C(acr(q));
-    }
-    const C r = C(j) + C(0.5), ir = C(1) / r;
-    const C g1 = I[I_G1 * A.plane], g2 = I[I_G2 * A.plane], g3 = I[I_G3 * A.plane];
-    const C cmu = (A.tau - C(0.5)) * C(1.0 / 3.0);
+    const C Sb = C(1.0 / 9.0) * M0, Hzb = C(1.0 / 3.0) * Mz, Hrb = C(1.0 / 3.0) * Mr;
+    const C d1r = I[I_G1 * A.plane] + I[I_G2 * A.plane], d3 = I[I_G3 * A.plane];
     const C muv = rho * cmu;
-    // S = -rho u_r / r
-    rb += -Sb * ur * ir;
-    urb += -Sb * rho * ir;
-    // H_z = (mu (g1 + g2) - rho u_r u_z) / r
-    C mvb = Hzb * (g1 + g2) * ir;
-    g1b = Hzb * muv * ir;
-    g2b = Hzb * muv * ir;
-    rb += -Hzb * ur * uz * ir;
-    urb += -Hzb * rho * uz * ir;
-    uzb += -Hzb * rho * ur * ir;
-    // H_r = (2 mu (g3 - u_r / r) - rho u_r^2) / r
-    mvb += Hrb * C(2) * (g3 - ur * ir) * ir;
-    g3b = Hrb * C(2) * muv * ir;
-    urb += Hrb * (-C(2) * muv * ir - C(2) * rho * ur) * ir;
-    rb += -Hrb * ur * ur * ir;
-    // mu = rho (tau - 1/2) / 3
-    rb += mvb * cmu;
+    // S = -rho u_r / r, H_z = (mu (g1 + g2) - rho u_r u_z) / r,
+    // H_r = (2 mu (g3 - u_r / r) - rho u_r^2) / r, mu = rho (tau - 1/2) / 3
+    const C hz = Hzb * irr, hr = Hrb * irr, sb = Sb * irr;
+    const C e3 = d3 - ur * irr;
+    const C mvb = hz * d1r + C(2) * hr * e3;
+    rb += mvb * cmu - ur * (sb + hz * uz + hr * ur);
+    urb = -rho * (sb + hz * uz + C(2) * hr * ur) - C(2) * hr * muv * irr;
+    uzb = -rho * hz * ur;
     tb += mvb * rho * C(1.0 / 3.0);
+    // transposed gradient stencils
+    const C* a = g1 + (ty + 2) * W + tx + 2;
+    uzb += d1_t(a, W) * C(1.0 / 12.0);
+    urb += (d1_t(a, 1) + d1_t(g3 + (ty + 2) * ATZ + tx, ATZ)) * C(1.0 / 12.0);
   }
-  A.rhob[o] = rb;
-  A.uzb[o] = uzb;
-  A.urb[o] = urb;
-  A.vzb[o] = vzb;
-  A.vrb[o] = vrb;
-  A.g1b[o] = g1b;
-  A.g2b[o] = g2b;
-  A.g3b[o] = g3b;
-  A.accT[o] += double(tb);
-}
-
-// ---- vel: transposed gradient stencils (u ghosts folded), adjoint of u and u^eq;
-// then (same site, no neighbours) the local adjoint of F_SC and F^gamma
-template <class C>
-__global__ void __launch_bounds__(ANT) adj_vel(Adj<C> A) {
-  constexpr int HR = 5;  // ghost rows -2, -1 and Nr, Nr + 1 reach two rows further
-  __shared__ Win<C, HR> w1, w2, w3;
-  const int k0 = blockIdx.x * ATZ, j0 = blockIdx.y * ATR;
-  const int k = k0 + (int)threadIdx.x % ATZ, j = j0 + (int)threadIdx.x / ATZ;
-  if (A.axisym) {
-    const bool near_edge = j0 < 2 || j0 + ATR > A.Nr - 2;
-    load_win<false>(w1, A.g1b, k0, j0, near_edge, A);
-    load_win<false>(w2, A.g2b, k0, j0, near_edge, A);
-    load_win<false>(w3, A.g3b, k0, j0, near_edge, A);
-    __syncthreads();
-  }
-  if (k >= A.Nz || j >= A.Nr) return;
-  const size_t o = (size_t)j * A.P + k;
-  C uzb = A.uzb[o], urb = A.urb[o];
-  if (A.axisym) {
-    const C szw = A.wall == AMLBM_WALL_NOSLIP ? C(-1) : C(1);
-    uzb += d1_tw<1>(w1, k, j, k0, j0);
-    urb += d1_tw<0>(w2, k, j, k0, j0) + d1_tw<1>(w3, k, j, k0, j0);
-    // ghost rows (depth 2) that mirror this row: u_z even / u_r odd at the axis;
-    // at the wall u_r odd and u_z even (free-slip) or odd (no-slip)
-    const int ga = -1 - j;
-    if (ga >= -2) {
-      uzb += d1_tw<1>(w1, k, ga, k0, j0);
-      urb -= d1_tw<0>(w2, k, ga, k0, j0) + d1_tw<1>(w3, k, ga, k0, j0);
-    }
-    const int gw = 2 * A.Nr - 1 - j;
-    if (gw <= A.Nr + 1) {
-      uzb += szw * d1_tw<1>(w1, k, gw, k0, j0);
-      urb -= d1_tw<0>(w2, k, gw, k0, j0) + d1_tw<1>(w3, k, gw, k0, j0);
-    }
-  }
-  const C* I = A.inter + o;
-  const C rho = I[I_RHO * A.plane], ir = C(1) / rho;
-  const C uz = I[I_UZ * A.plane], ur = I[I_UR * A.plane], vz = I[I_VZ * A.plane],
-          vr = I[I_VR * A.plane], Fz = I[I_FZ * A.plane], Fr = I[I_FR * A.plane];
-  const C vzb = A.vzb[o], vrb = A.vrb[o];
+  // u = (j + F/2)/rho and u^eq = (j + tau F)/rho
+  const C ir = C(1) / rho;
+  const C Fz = I[I_FZ * A.plane], Fr = I[I_FR * A.plane];
   A.jzb[o] = (uzb + vzb) * ir;
   A.jrb[o] = (urb + vrb) * ir;
   const C Fzb = (C(0.5) * uzb + A.tau * vzb) * ir, Frb = (C(0.5) * urb + A.tau * vrb) * ir;
-  A.Fzb[o] = Fzb;
-  A.Frb[o] = Frb;
-  A.rhob[o] += -(uzb * uz + urb * ur + vzb * vz + vrb * vr) * ir + Fzb * A.gz;
-  double tacc = double((vzb * Fz + vrb * Fr) * ir);
+  A.rhob[o] = rb - (uzb * uz + urb * ur + vzb * vz + vrb * vr) * ir + Fzb * A.gz;
   // F_SC = -G psi s
-  const C psi = I[I_PSI * A.plane], sz = I[I_SZ * A.plane], sr = I[I_SR * A.plane];
-  C pb = -A.G * (Fzb * sz + Frb * sr);
-  double gb = double(-psi * (Fzb * sz + Frb * sr));
+  const C psi = I[I_PSI * A.plane];
+  const C sf = Fzb * I[I_SZ * A.plane] + Frb * I[I_SR * A.plane];
+  C pb = -A.G * sf;
+  double gb = double(-psi * sf);
   A.qz[o] = -A.G * psi * Fzb;
   A.qr[o] = -A.G * psi * Frb;
-  C dzrb = C(0), drrb = C(0), drdb = C(0);
   if (A.axisym) {
-    const C irr = C(1) / (C(j) + C(0.5));
-    const C Dr = I[I_DR * A.plane], Drr = I[I_DRR * A.plane], Dzr = I[I_DZR * A.plane];
-    const C gf = -A.G * C(1.0 / 18.0);
-    const C t = Fzb * Dzr * irr + Frb * (Drr * irr - Dr * irr * irr);
+    const C gf = -A.G * C(1.0 / 18.0), gi = gf * psi * irr;
+    const C t = irr * (Fzb * I[I_DZR * A.plane] + Frb * (I[I_DRR * A.plane] - I[I_DR * A.plane] * irr));
     pb += gf * t;
     gb += double(-psi * t * C(1.0 / 18.0));
-    dzrb = gf * psi * Fzb * irr;
-    drrb = gf * psi * Frb * irr;
-    drdb = -gf * psi * Frb * irr * irr;
+    A.dzrb[o] = gi * Fzb;
+    A.drrb[o] = gi * Frb;
+    A.drdb[o] = -gi * Frb * irr;
   }
   A.psib[o] = pb;
-  A.dzrb[o] = dzrb;
-  A.drrb[o] = drrb;
-  A.drdb[o] = drdb;
   A.accG[o] += gb;
-  A.accT[o] += tacc;
+  A.accT[o] += double(tb) + double((vzb * Fz + vrb * Fr) * ir);
+  pdl_trigger();
 }
 
-
-// ---- deriv: transposed 1D d_z (into the 1D d_r field) and isotropic d_r (into
-// the padded d_r psi field, rows -2 .. Nr+1); tiles of the padded rows
-template <class C>
-__global__ void __launch_bounds__(ANT) adj_deriv(Adj<C> A) {
-  __shared__ Win<C, 2> wr;             // d_rr psi adjoint, padded rows jp0 - 2 .. jp0 + ATR + 1
-  __shared__ C wd[ATR * (ATZ + 4)];    // d_zr psi adjoint, rows jp0 .. jp0 + ATR - 1
-  const int k0 = blockIdx.x * ATZ, jp0 = -2 + (int)blockIdx.y * ATR;
-  load_win<false>(wr, A.drrb, k0, jp0, true, A);
-  for (int i = threadIdx.x; i < ATR * (ATZ + 4); i += ANT) {
-    const int rr = i / (ATZ + 4), cc = i - rr * (ATZ + 4);
-    const int y = jp0 + rr;
-    wd[i] = (y >= 0 && y < A.Nr) ? A.dzrb[(size_t)y * A.P + wz(k0 - 2 + cc, A.Nz)] : C(0);
+template <class C, int BR>
+__global__ void __launch_bounds__(ATZ * BR) adj_psi(Adj<C> A) {
+  constexpr int NT = ATZ * BR;
+  constexpr int RZ = ATZ + 8, RR = BR + 8;  // adjoint of d_rr psi, even in r
+  constexpr int DZ = ATZ + 4, DR = BR + 4;  // adjoint of d_r psi, odd in r
+  constexpr int QZ = ATZ + 2, QR = BR + 2;  // adjoints of the Shan-Chen sums: z even, r odd
+  __shared__ C srr[RR * RZ], szr[DR * DZ], sdr[DR * DZ], seb[DR * ATZ], sqz[QR * QZ], sqr[QR * QZ];
+  __shared__ int s_col[RZ], s_off[RR];  // columns and row offsets of the tile + 4 (-1: beyond the ghost rows)
+  const int k0 = blockIdx.x * ATZ, j0 = blockIdx.y * BR;
+  const int tx = (int)threadIdx.x % ATZ, ty = (int)threadIdx.x / ATZ, k = k0 + tx, j = j0 + ty;
+  const bool in = k < A.Nz && j < A.Nr, ax = A.axisym != 0;
+  const size_t o = (size_t)(in ? j : 0) * A.P + (in ? k : 0);
+  for (int i = threadIdx.x; i < RZ; i += NT) s_col[i] = wz(k0 - 4 + i, A.Nz);
+  if (threadIdx.x < RR) {
+    const int m = mirror_row(j0 - 4 + (int)threadIdx.x, A.Nr);
+    s_off[threadIdx.x] = m < 0 || m >= A.Nr ? -1 : m * A.P;
   }
   __syncthreads();
-  const int tx = (int)threadIdx.x % ATZ, ty = (int)threadIdx.x / ATZ;
-  const int k = k0 + tx, jp = jp0 + ty;
-  if (k >= A.Nz || jp > A.Nr + 1) return;
-  if (jp >= 0 && jp < A.Nr) {
-    const C* d = wd + ty * (ATZ + 4) + tx + 2;  // column k
-    const C e = (C(8) * (d[-1] - d[1]) - (d[-2] - d[2])) * C(1.0 / 12.0);
-    A.eb[(size_t)jp * A.P + k] = e;
-  }
-  C v = iso_tw<1>(wr, k, jp, k0, jp0);
-  if (jp >= 0 && jp < A.Nr) v += A.drdb[(size_t)jp * A.P + k];
-  A.drpb[(size_t)(jp + 2) * A.P + k] = v;
-}
-
-// psi adjoint at the (possibly ghost) position (k, y): transposed Shan-Chen
-// neighbour sum, 1D d_r and isotropic d_r, from the windows of q_z, q_r, the 1D
-// d_r adjoint e and the padded d_r psi adjoint.
-template <class C, int HR>
-__device__ __forceinline__ C psi_pad_adj(int k, int y, int k0, int j0, const Win<C, HR>& qz,
-                                         const Win<C, HR>& qr, const Win<C, HR>& eb,
-                                         const Win<C, HR>& dp, bool axisym) {
-  C s = C(0);
+  pdl_wait();
+  C mu[9];
+  if (in) {
 #pragma unroll
-  for (int i = 1; i < 9; ++i) {
-    const C w = C(aw(i));
-    if (acz(i)) s += w * C(acz(i)) * wat(qz, k - acz(i), y - acr(i), k0, j0);
-    if (acr(i)) s += w * C(acr(i)) * wat(qr, k - acz(i), y - acr(i), k0, j0);
+    for (int q = 0; q < 9; ++q) mu[q] = arrived(A, q, k, j);
   }
-  if (axisym) {
-    s += (C(8) * (wat(eb, k, y - 1, k0, j0) - wat(eb, k, y + 1, k0, j0)) -
-          (wat(eb, k, y - 2, k0, j0) - wat(eb, k, y + 2, k0, j0))) * C(1.0 / 12.0);
-    s += iso_tw<1>(dp, k, y, k0, j0);
-  }
-  return s;
-}
-
-// ---- final: psi ghosts folded (even mirrors, depth 4), d psi / d rho, lambda^n
-template <class C>
-__global__ void __launch_bounds__(ANT) adj_final(Adj<C> A) {
-  constexpr int HR = 9;  // ghost rows down to -4 and up to Nr + 3, read at distance 2
-  __shared__ Win<C, HR> wqz, wqr, web, wdp;
-  const int k0 = blockIdx.x * ATZ, j0 = blockIdx.y * ATR;
-  const int k = k0 + (int)threadIdx.x % ATZ, j = j0 + (int)threadIdx.x / ATZ;
-  const bool near_edge = j0 < 4 || j0 + ATR > A.Nr - 4;
-  load_win<false>(wqz, A.qz, k0, j0, near_edge, A);
-  load_win<false>(wqr, A.qr, k0, j0, near_edge, A);
-  if (A.axisym) {
-    load_win<false>(web, A.eb, k0, j0, near_edge, A);
-    load_win<true>(wdp, A.drpb, k0, j0, near_edge, A);
+  for_region<NT, QR, QZ>([&](int lr, int lc) {
+    const int off = s_off[lr + 3], row = j0 - 1 + lr;
+    if (off < 0) return;
+    const int p = off + s_col[lc + 3];
+    const C r = A.qr[p];
+    sqz[lr * QZ + lc] = A.qz[p];
+    sqr[lr * QZ + lc] = row < 0 || row >= A.Nr ? -r : r;
+  });
+  if (ax) {
+    for_region<NT, RR, RZ>([&](int lr, int lc) {
+      const int off = s_off[lr];
+      if (off >= 0) srr[lr * RZ + lc] = A.drrb[off + s_col[lc]];
+    });
+    for_region<NT, DR, DZ>([&](int lr, int lc) {
+      const int off = s_off[lr + 2];
+      if (off < 0) return;
+      const int p = off + s_col[lc + 2];
+      szr[lr * DZ + lc] = A.dzrb[p];
+      sdr[lr * DZ + lc] = A.drdb[p];
+    });
+    __syncthreads();
+    for_region<NT, DR, DZ>([&](int lr, int lc) {
+      const int row = j0 - 2 + lr;
+      const bool ghost = row < 0 || row >= A.Nr;
+      // a mirrored row's transpose has the mirrored sign of the row's own
+      const C d = iso_t(srr + (lr + 2) * RZ + lc + 2, RZ) * C(1.0 / 36.0);
+      const C own = sdr[lr * DZ + lc];
+      sdr[lr * DZ + lc] = ghost ? d - own : d + own;
+      if (lc >= 2 && lc < ATZ + 2) {
+        const C e = d1_t(szr + lr * DZ + lc, 1) * C(1.0 / 12.0);
+        seb[lr * ATZ + lc - 2] = ghost ? -e : e;
+      }
+    });
   }
   __syncthreads();
-  if (k >= A.Nz || j >= A.Nr) return;
-  const size_t o = (size_t)j * A.P + k;
-  const bool ax = A.axisym != 0;
-  C pb = A.psib[o] + psi_pad_adj(k, j, k0, j0, wqz, wqr, web, wdp, ax);
-  const int ga = -1 - j;
-  if (ga >= -4) pb += psi_pad_adj(k, ga, k0, j0, wqz, wqr, web, wdp, ax);
-  const int gw = 2 * A.Nr - 1 - j;
-  if (gw <= A.Nr + 3) pb += psi_pad_adj(k, gw, k0, j0, wqz, wqr, web, wdp, ax);
-  const C rho = A.inter[I_RHO * A.plane + o];
-  const C rb = A.rhob[o] + pb * exp(-rho * A.inv_rho0);
-  const C jzb = A.jzb[o], jrb = A.jrb[o];
+  if (in) {
+    const C* z = sqz + (ty + 1) * QZ + tx + 1;
+    const C* r = sqr + (ty + 1) * QZ + tx + 1;
+    C pb = A.psib[o] +
+           C(1.0 / 9.0) * ((z[-1] - z[1]) + (r[-QZ] - r[QZ])) +
+           C(1.0 / 36.0) * (((z[-QZ - 1] - z[QZ + 1]) + (z[QZ - 1] - z[-QZ + 1])) +
+                            ((r[-QZ - 1] - r[QZ + 1]) + (r[-QZ + 1] - r[QZ - 1])));
+    if (ax) {
+      pb += d1_t(seb + (ty + 2) * ATZ + tx, ATZ) * C(1.0 / 12.0);
+      pb += iso_t(sdr + (ty + 2) * DZ + tx + 2, DZ) * C(1.0 / 36.0);
+    }
+    // d psi / d rho = exp(-rho / rho0); in FP64 1 - psi / rho0 (an exp is 20 FP64 operations)
+    C dpsi;
+    if constexpr (sizeof(C) == 8) dpsi = C(1) - A.inter[I_PSI * A.plane + o] * A.inv_rho0;
+    else dpsi = exp(-A.inter[I_RHO * A.plane + o] * A.inv_rho0);
+    const C rb = A.rhob[o] + pb * dpsi;
+    const C jzb = A.jzb[o], jrb = A.jrb[o];
 #pragma unroll
-  for (int q = 0; q < 9; ++q)
-    A.lam_out[q * A.plane + o] =
-        (C(1) - A.omega) * A.mu[q * A.plane + o] + rb + C(acz(q)) * jzb + C(acr(q)) * jrb;
+    for (int q = 0; q < 9; ++q)
+      A.lam_out[q * A.plane + o] = (C(1) - A.omega) * mu[q] + (rb + C(acz(q)) * jzb + C(acr(q)) * jrb);
+  }
+  pdl_trigger();
 }
 
 // ---- the differentiable initial drop and its adjoint
+// The Legendre polynomials of all amplitudes come from one upward recurrence,
+// P_{m+1} = ((2m + 1) x P_m - m P_{m-1}) / (m + 1), the division as a product with a
+// reciprocal from the host (one recurrence per amplitude and an FP64 division per degree
+// took 295 us for the drop and 602 us for its adjoint on 512 x 128 with 16 amplitudes).
+constexpr int kMaxDegree = 64;
 struct DropMap {
   int Nz, Nr, l0, namp;
   double zc, R, w, rho_l, rho_v;
   double amp[32];
+  double inv[kMaxDegree];  // 1 / m
 };
 
-__device__ double legendre_d(int l, double x) {
-  double p0 = 1.0, p1 = x;
-  if (l == 0) return p0;
-  for (int m = 1; m < l; ++m) {
-    const double p2 = ((2.0 * m + 1.0) * x * p1 - m * p0) / (m + 1);
-    p0 = p1;
-    p1 = p2;
-  }
-  return p1;
+// P_m(x) and P_{m+1}(x), advanced by one degree from m.
+__device__ __forceinline__ void legendre_next(const DropMap& M, int m, double x, double& p, double& next) {
+  const double q = ((2 * m + 3) * x * next - (m + 1) * p) * (m + 2 < kMaxDegree ? M.inv[m + 2] : 1.0 / (m + 2));
+  p = next;
+  next = q;
+}
+__device__ __forceinline__ void legendre_start(const DropMap& M, double x, double& p, double& next) {
+  p = 1.0;
+  next = x;
+  for (int m = 0; m < M.l0; ++m) legendre_next(M, m, x, p, next);
 }
 
 __global__ void drop_kernel(DropMap M, double* rho) {
@@ -428,20 +400,26 @@ __global__ void drop_kernel(DropMap M, double* rho) {
   if (n >= M.Nz * M.Nr) return;
   const int j = n / M.Nz, k = n - j * M.Nz;
   const double dz = k - M.zc, r = j + 0.5, d = sqrt(dz * dz + r * r), ct = dz / d;
-  double s = 0.0;
-  for (int m = 0; m < M.namp; ++m) s += M.amp[m] * legendre_d(M.l0 + m, ct);
+  double s = 0.0, p, next;
+  legendre_start(M, ct, p, next);
+  for (int m = 0; m < M.namp; ++m) {
+    s += M.amp[m] * p;
+    legendre_next(M, M.l0 + m, ct, p, next);
+  }
   const double Rs = M.R * (1.0 + s);
   rho[n] = M.rho_v + 0.5 * (M.rho_l - M.rho_v) * (1.0 - tanh((d - Rs) / M.w));
 }
 
 constexpr int RED_NT = 256;
-// per-block sums of sum_x rho_bar(x) d rho(x) / d a_m, rho_bar = sum_i W_i lambda^0_i
-template <class C>
+// per-block sums of sum_x rho_bar(x) d rho(x) / d a_m, rho_bar = sum_i W_i lambda^0_i;
+// N >= namp amplitudes in registers
+template <class C, int N>
 __global__ void __launch_bounds__(RED_NT) drop_adj_kernel(DropMap M, const C* lam, size_t plane,
                                                           int P, double* partials) {
-  __shared__ double red[RED_NT];
-  double acc[32];
-  for (int m = 0; m < M.namp; ++m) acc[m] = 0.0;
+  __shared__ double red[RED_NT / 32][N];
+  double acc[N];
+#pragma unroll
+  for (int m = 0; m < N; ++m) acc[m] = 0.0;
   for (int n = blockIdx.x * RED_NT + threadIdx.x; n < M.Nz * M.Nr; n += gridDim.x * RED_NT) {
     const int j = n / M.Nz, k = n - j * M.Nz;
     const size_t o = (size_t)j * P + k;
@@ -449,21 +427,37 @@ __global__ void __launch_bounds__(RED_NT) drop_adj_kernel(DropMap M, const C* la
 #pragma unroll
     for (int q = 0; q < 9; ++q) rb += aw(q) * double(lam[q * plane + o]);
     const double dz = k - M.zc, r = j + 0.5, d = sqrt(dz * dz + r * r), ct = dz / d;
-    double s = 0.0;
-    for (int m = 0; m < M.namp; ++m) s += M.amp[m] * legendre_d(M.l0 + m, ct);
-    const double X = (d - M.R * (1.0 + s)) / M.w, sh = 1.0 / cosh(X);
-    const double dr_dRs = 0.5 * (M.rho_l - M.rho_v) * sh * sh / M.w;
-    for (int m = 0; m < M.namp; ++m) acc[m] += rb * dr_dRs * M.R * legendre_d(M.l0 + m, ct);
-  }
-  for (int m = 0; m < M.namp; ++m) {
-    red[threadIdx.x] = acc[m];
-    __syncthreads();
-    for (int s = RED_NT / 2; s > 0; s >>= 1) {
-      if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-      __syncthreads();
+    double s = 0.0, p, next;
+    legendre_start(M, ct, p, next);
+    const double p0 = p, next0 = next;
+    for (int m = 0; m < M.namp; ++m) {
+      s += M.amp[m] * p;
+      legendre_next(M, M.l0 + m, ct, p, next);
     }
-    if (threadIdx.x == 0) partials[blockIdx.x * 32 + m] = red[0];
-    __syncthreads();
+    const double X = (d - M.R * (1.0 + s)) / M.w, sh = 1.0 / cosh(X);
+    const double c = rb * (0.5 * (M.rho_l - M.rho_v) * sh * sh / M.w) * M.R;
+    p = p0;
+    next = next0;
+#pragma unroll
+    for (int m = 0; m < N; ++m) {
+      if (m >= M.namp) break;
+      acc[m] += c * p;
+      legendre_next(M, M.l0 + m, ct, p, next);
+    }
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int m = 0; m < N; ++m) {
+    if (m >= M.namp) break;
+    double v = acc[m];
+    for (int w = 16; w > 0; w >>= 1) v += __shfl_xor_sync(0xffffffffu, v, w);
+    if (lane == 0) red[warp][m] = v;
+  }
+  __syncthreads();
+  if ((int)threadIdx.x < M.namp) {
+    double v = 0.0;
+    for (int w = 0; w < RED_NT / 32; ++w) v += red[w][threadIdx.x];
+    partials[blockIdx.x * 32 + threadIdx.x] = v;
   }
 }
 
@@ -493,20 +487,14 @@ __global__ void __launch_bounds__(RED_NT) sum2_kernel(const double* a, const dou
   }
 }
 
-// lambda^T = dJ/df_i(x) = dJ/drho(x) for every i
+// lambda^T = dJ/df_i(x) = dJ/drho(x) for every i; coef: the objective's constant factor
 template <class C>
-__global__ void seed_kernel(int kind, int Nz, int Nr, int P, size_t plane, double zc, double objR,
-                            double rho_l, double rho_v, int kstar, double a2_or_J, C* lam) {
+__global__ void seed_kernel(int kind, int Nz, int Nr, int P, size_t plane, double zc, int kstar, double coef, C* lam) {
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= Nz * Nr) return;
   const int j = n / Nz, k = n - j * Nz;
-  const double pi = 3.14159265358979323846, r = j + 0.5, dz = k - zc;
-  double s;
-  if (kind == AMLBM_OBJ_A2SQ)
-    s = 2.0 * a2_or_J * 5.0 / (4.0 * pi * pow(objR, 5.0)) * 2.0 * pi * r * (dz * dz - 0.5 * r * r) /
-        (rho_l - rho_v);
-  else
-    s = k == kstar ? r / ((rho_l - rho_v) * a2_or_J) : 0.0;
+  const double r = j + 0.5, dz = k - zc;
+  const double s = kind == AMLBM_OBJ_A2SQ ? coef * (r * (dz * dz - 0.5 * r * r)) : k == kstar ? coef * r : 0.0;
 #pragma unroll
   for (int q = 0; q < 9; ++q) lam[q * plane + (size_t)j * P + k] = C(s);
 }
@@ -529,14 +517,14 @@ namespace {
 
 struct AdjLayout {
   size_t total = 0;
-  size_t ckpt = 0, seg = 0, lam = 0, inter = 0, fstar = 0, mu = 0, arr = 0, drp = 0, acc = 0, rho0 = 0,
+  size_t ckpt = 0, seg = 0, lam = 0, inter = 0, fstar = 0, arr = 0, acc = 0, rho0 = 0,
          red = 0, descs = 0, tiles = 0;
   int nck = 0, nseg = 0, ntiles = 0, nred = 0;
   int nbuf = 1;            // segment buffers: two when there are several segments
   size_t state_elems = 0;  // 10 planes (f and psi)
 };
 
-constexpr int kAdjArrays = 19;
+constexpr int kAdjArrays = 9;
 
 size_t al(size_t x) { return (x + 255) / 256 * 256; }
 
@@ -560,9 +548,7 @@ AdjLayout adj_layout(const amlbm::CtxInfo& ci, const amlbm_adjoint_problem& p) {
   L.lam = take(2 * 9 * plane * cb);
   L.inter = take((size_t)L.nbuf * L.nseg * amlbm::I_COUNT * plane * cb);
   L.fstar = take(ci.storage == AMLBM_STORE_F64 ? 9 * plane * cb : 0);
-  L.mu = take(9 * plane * cb);
   L.arr = take((size_t)kAdjArrays * plane * cb);
-  L.drp = take((size_t)(ci.Nr + 4) * ci.host.P * cb);
   L.acc = take(2 * plane * sizeof(double));
   L.rho0 = take((size_t)ci.Nz * ci.Nr * sizeof(double));
   const int nblk = amlbm::diag_blocks(ci.Nz, ci.Nr);
@@ -647,6 +633,7 @@ int run(amlbm_ctx* ctx, const amlbm_adjoint_problem* p, void* ws, size_t ws_byte
     M.Nz = Nz; M.Nr = Nr; M.l0 = p->l0; M.namp = p->n_amps;
     M.zc = p->zc; M.R = p->R; M.w = p->w; M.rho_l = p->rho_l; M.rho_v = p->rho_v;
     for (int m = 0; m < p->n_amps; ++m) M.amp[m] = p->amps[m];
+    for (int m = 1; m < kMaxDegree; ++m) M.inv[m] = 1.0 / m;
 
     // forward: initial drop, T steps, states every ckpt_every steps
     drop_kernel<<<nb, 256, 0, s>>>(M, rho_init);
@@ -681,9 +668,11 @@ int run(amlbm_ctx* ctx, const amlbm_adjoint_problem* p, void* ws, size_t ws_byte
       }
       if (J) *J = Jv;
       if (!adjoint) goto done;
-      seed_kernel<C><<<nb, 256, 0, s>>>(p->objective, Nz, Nr, P, plane, p->zc, p->obj_R, p->rho_l,
-                                        p->rho_v, p->kstar, p->objective == AMLBM_OBJ_A2SQ ? a2 : Jv,
-                                        lam[0]);
+      // J = a2^2, a2 = a2_norm sum 2 pi r phi (dz^2 - r^2/2); or J = sqrt(2 sum r phi)
+      const double coef = p->objective == AMLBM_OBJ_A2SQ
+                              ? 2.0 * a2 * a2_norm(p->obj_R) * 2.0 * 3.14159265358979323846 / (p->rho_l - p->rho_v)
+                              : 1.0 / ((p->rho_l - p->rho_v) * Jv);
+      seed_kernel<C><<<nb, 256, 0, s>>>(p->objective, Nz, Nr, P, plane, p->zc, p->kstar, coef, lam[0]);
       ADJ_CK(cudaGetLastError());
     }
     // descriptors of the segment slots (tiled by inter_tile): descriptor q of buffer b
@@ -713,22 +702,19 @@ int run(amlbm_ctx* ctx, const amlbm_adjoint_problem* p, void* ws, size_t ws_byte
       Adj<C> A;
       A.Nz = Nz; A.Nr = Nr; A.P = P; A.wall = ci.host.wall; A.axisym = ci.host.axisym;
       A.plane = plane;
-      A.tau = C(ci.host.tau); A.omega = C(1) / A.tau; A.G = C(ci.host.G); A.rho0 = C(ci.host.rho0);
+      A.tau = C(ci.host.tau); A.omega = C(1) / A.tau; A.G = C(ci.host.G);
       A.gz = C(ci.host.gz);
       A.inv_rho0 = C(1.0 / ci.host.rho0);
-      A.mu = reinterpret_cast<C*>(base + L.mu);
       C* arr = reinterpret_cast<C*>(base + L.arr);
-      C** fields[kAdjArrays] = {&A.rhob, &A.uzb, &A.urb, &A.vzb, &A.vrb, &A.g1b, &A.g2b, &A.g3b, &A.jzb,
-                                &A.jrb, &A.Fzb, &A.Frb, &A.psib, &A.qz, &A.qr, &A.dzrb, &A.drrb, &A.drdb,
-                                &A.eb};
+      C** fields[kAdjArrays] = {&A.rhob, &A.jzb, &A.jrb, &A.psib, &A.qz, &A.qr, &A.dzrb, &A.drrb, &A.drdb};
       for (int q = 0; q < kAdjArrays; ++q) *fields[q] = arr + (size_t)q * plane;
-      A.drpb = reinterpret_cast<C*>(base + L.drp);
       A.accG = reinterpret_cast<double*>(base + L.acc);
       A.accT = A.accG + plane;
       const InstDesc* d_seg = reinterpret_cast<const InstDesc*>(base + L.descs);
       const int* d_tiles = reinterpret_cast<const int*>(base + L.tiles);
-      const dim3 tgrid((Nz + ATZ - 1) / ATZ, (Nr + ATR - 1) / ATR);
-      const dim3 dgrid((Nz + ATZ - 1) / ATZ, (Nr + 4 + ATR - 1) / ATR);  // padded rows -2 .. Nr + 1
+      // 32 x 8 tiles, or 32 x 4 where those would leave SMs without one
+      const int gz = (Nz + ATZ - 1) / ATZ;
+      const bool low = gz * ((Nr + 7) / 8) < 152;
       C* inter_seg = reinterpret_cast<C*>(base + L.inter);
       const size_t iseg = (size_t)I_COUNT * plane;
       // Segment buffer b: states, intermediates and step descriptors.
@@ -754,48 +740,33 @@ int run(amlbm_ctx* ctx, const amlbm_adjoint_problem* p, void* ws, size_t ws_byte
           B.f = seg_of(b) + (size_t)q * L.state_elems;
           B.lam_in = lam[c];
           B.lam_out = lam[c ^ 1];
-          adj_post<C><<<tgrid, ANT, 0, st>>>(B);
-          adj_vel<C><<<tgrid, ANT, 0, st>>>(B);
-          adj_deriv<C><<<dgrid, ANT, 0, st>>>(B);
-          adj_final<C><<<tgrid, ANT, 0, st>>>(B);
+          const dim3 grid(gz, low ? (Nr + 3) / 4 : (Nr + 7) / 8);
+          cudaError_t e = low ? launch_pdl(adj_local<C, 4>, grid, ATZ * 4, 0, st, B)
+                              : launch_pdl(adj_local<C, 8>, grid, ATZ * 8, 0, st, B);
+          if (e == cudaSuccess)
+            e = low ? launch_pdl(adj_psi<C, 4>, grid, ATZ * 4, 0, st, B)
+                    : launch_pdl(adj_psi<C, 8>, grid, ATZ * 8, 0, st, B);
+          if (e != cudaSuccess) return e;
           c ^= 1;
         }
-        return cudaGetLastError();
+        return cudaSuccess;
       };
       // Segments run from the last to the first.  The recompute of segment m - 1
       // (on stream rs, into the other buffer) does not depend on the backward
       // sweep of segment m (on s), so the two overlap: each is a few hundred CTAs
       // and leaves most of the GPU idle.  Events order each recompute after the
       // backward sweep that last read its buffer, and each backward sweep after
-      // its recompute.  Full segments issue the same launches every time, so after
-      // one direct run each part is replayed from a captured CUDA graph (keyed by
-      // buffer, and by the starting lambda buffer for the backward part).  Any
-      // failure of the graph machinery falls back to direct launches.
-      cudaStream_t rs = nullptr, gs = nullptr;
+      // its recompute.  (The host issues the four launches of a step, three in FP32, faster
+      // than the GPU runs them; capturing each call's segments into graphs cost more than
+      // it saved.)
+      cudaStream_t rs = nullptr;
       cudaEvent_t ev0 = nullptr, evR[2] = {nullptr, nullptr}, evB[2] = {nullptr, nullptr};
-      cudaGraphExec_t gR[2] = {nullptr, nullptr}, gB[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
       bool usedB[2] = {false, false};
       bool streams_ok = cudaStreamCreateWithFlags(&rs, cudaStreamNonBlocking) == cudaSuccess &&
                         cudaEventCreateWithFlags(&ev0, cudaEventDisableTiming) == cudaSuccess;
       for (int b = 0; b < 2 && streams_ok; ++b)
         streams_ok = cudaEventCreateWithFlags(&evR[b], cudaEventDisableTiming) == cudaSuccess &&
                      cudaEventCreateWithFlags(&evB[b], cudaEventDisableTiming) == cudaSuccess;
-      bool use_graph = streams_ok && cudaStreamCreateWithFlags(&gs, cudaStreamNonBlocking) == cudaSuccess;
-      bool r_direct = false, b_direct = false;  // a full segment has run directly
-      // capture `fn` (which launches on its stream argument) into *gx
-      auto capture = [&](cudaGraphExec_t* gx, auto fn) {
-        cudaGraph_t g = nullptr;
-        cudaError_t e = cudaStreamBeginCapture(gs, cudaStreamCaptureModeThreadLocal);
-        const cudaError_t e1 = e == cudaSuccess ? fn(gs) : e;
-        if (e == cudaSuccess) e = cudaStreamEndCapture(gs, &g);
-        if (e == cudaSuccess && e1 == cudaSuccess) e = cudaGraphInstantiate(gx, g, 0);
-        if (g) cudaGraphDestroy(g);
-        if (e != cudaSuccess || e1 != cudaSuccess) {
-          use_graph = false;
-          *gx = nullptr;
-          cudaGetLastError();  // the direct path reports real errors
-        }
-      };
       cudaStream_t rstream = streams_ok ? rs : s;  // without a second stream, no overlap
 #define SEG_CK(call)                                                                          \
   {                                                                                           \
@@ -815,15 +786,7 @@ int run(amlbm_ctx* ctx, const amlbm_adjoint_problem* p, void* ws, size_t ws_byte
         cudaError_t e = cudaMemcpyAsync(seg_of(b), ckpt + (size_t)m * L.state_elems, SB,
                                         cudaMemcpyDeviceToDevice, rstream);
         if (e != cudaSuccess) return e;
-        const bool full = len == p->ckpt_every;
-        if (use_graph && r_direct && full) {
-          if (!gR[b]) capture(&gR[b], [&](cudaStream_t st) { return recompute(len, b, st); });
-          if (use_graph) e = cudaGraphLaunch(gR[b], rstream);
-          else e = recompute(len, b, rstream);
-        } else {
-          e = recompute(len, b, rstream);
-          if (full) r_direct = true;
-        }
+        e = recompute(len, b, rstream);
         if (e == cudaSuccess && streams_ok) e = cudaEventRecord(evR[b], rstream);
         return e;
       };
@@ -841,15 +804,7 @@ int run(amlbm_ctx* ctx, const amlbm_adjoint_problem* p, void* ws, size_t ws_byte
           // stream it would have to wait for this backward sweep, so it is issued after it
           if (m >= 1 && streams_ok) SEG_CK(issue_recompute(m - 1, (m - 1) % L.nbuf));
           if (streams_ok) SEG_CK(cudaStreamWaitEvent(s, evR[b], 0));
-          const bool full = len == p->ckpt_every;
-          if (use_graph && b_direct && full) {
-            if (!gB[b][cur]) capture(&gB[b][cur], [&](cudaStream_t st) { return backward(len, b, cur, st); });
-            if (use_graph) SEG_CK(cudaGraphLaunch(gB[b][cur], s))
-            else SEG_CK(backward(len, b, cur, s))
-          } else {
-            SEG_CK(backward(len, b, cur, s));
-            if (full) b_direct = true;
-          }
+          SEG_CK(backward(len, b, cur, s));
           if (streams_ok) {
             SEG_CK(cudaEventRecord(evB[b], s));
             usedB[b] = true;
@@ -858,26 +813,21 @@ int run(amlbm_ctx* ctx, const amlbm_adjoint_problem* p, void* ws, size_t ws_byte
           if (len & 1) cur ^= 1;
         }
       } while (false);
-      // graphs run on s and rs: let them finish before their executables go
       if (rs) cudaStreamSynchronize(rs);
-      if (gs) cudaStreamSynchronize(gs);
       cudaStreamSynchronize(s);
-      for (auto& g : gR)
-        if (g) cudaGraphExecDestroy(g);
-      for (auto& row : gB)
-        for (auto& g : row)
-          if (g) cudaGraphExecDestroy(g);
       for (auto* ev : {ev0, evR[0], evR[1], evB[0], evB[1]})
         if (ev) cudaEventDestroy(ev);
       if (rs) cudaStreamDestroy(rs);
-      if (gs) cudaStreamDestroy(gs);
 #undef SEG_CK
       if (rc) goto done;
       // parameter gradients (FP64, fixed order)
       sum2_kernel<<<L.nred, RED_NT, 0, s>>>(A.accG, A.accT, Nz, Nr, P, redbuf);
       ADJ_CK(cudaGetLastError());
       if (p->n_amps > 0) {
-        drop_adj_kernel<C><<<L.nred, RED_NT, 0, s>>>(M, lam[cur], plane, P, redbuf + 2 * L.nred);
+        double* part = redbuf + 2 * L.nred;
+        if (p->n_amps <= 4) drop_adj_kernel<C, 4><<<L.nred, RED_NT, 0, s>>>(M, lam[cur], plane, P, part);
+        else if (p->n_amps <= 16) drop_adj_kernel<C, 16><<<L.nred, RED_NT, 0, s>>>(M, lam[cur], plane, P, part);
+        else drop_adj_kernel<C, 32><<<L.nred, RED_NT, 0, s>>>(M, lam[cur], plane, P, part);
         ADJ_CK(cudaGetLastError());
       }
       red.resize((size_t)L.nred * 34);

@@ -19,9 +19,9 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <class... K, class... A>
-cudaError_t launch_pdl(void (*kernel)(K...), int grid, int block, size_t smem, cudaStream_t s, A... args) {
+cudaError_t launch_pdl(void (*kernel)(K...), dim3 grid, int block, size_t smem, cudaStream_t s, A... args) {
   cudaLaunchConfig_t c = {};
-  c.gridDim = dim3((unsigned)grid);
+  c.gridDim = grid;
   c.blockDim = dim3((unsigned)block);
   c.dynamicSmemBytes = smem;
   c.stream = s;
