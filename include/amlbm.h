@@ -337,7 +337,8 @@ typedef struct amlbm_instance {
  * the fused update with two adjacent z-sites per thread (vector loads and
  * stores, stencil taps shared by the pair), on tiles, or for the FP32-arithmetic
  * forms with tile_z = 48 on strips: one warp marches over tile_r rows of 48
- * columns (a lattice of at most 64 columns is one strip); it takes periodic lattices on the
+ * columns (a lattice of at most 64 columns is one strip); the library's own choice
+ * for FP32 storage runs lattices of odd width on strips too.  A request for it takes periodic lattices on the
  * axis with an even Nz, a free-slip or no-slip outer wall, the source at the
  * departure site (AMLBM_SRC_LOCAL) and either forcing, and 9 x pitch x Nr below
  * 2^31 elements.  All three give bit-identical states. */

@@ -96,15 +96,16 @@ bool bounded(const amlbm_bc& bc) {
 // A lattice the pair schedule takes: periodic in z with an even Nz, the axis
 // below row 0, a reflecting or bounce-back outer wall, the source at the
 // departure site, and element offsets of all nine planes within 32 bits.
-bool pair_ok(const amlbm_instance& I) {
+// (The strips also take an odd Nz in FP32 storage, which the library chooses by itself.)
+bool pair_ok(const amlbm_instance& I, bool odd = false) {
   return I.bc.z_bc == AMLBM_Z_PERIODIC && I.bc.r_lo == AMLBM_RLO_AXIS &&
          (I.bc.wall_r == AMLBM_WALL_FREESLIP || I.bc.wall_r == AMLBM_WALL_NOSLIP) &&
-         I.bc.src_mode == AMLBM_SRC_LOCAL && I.Nz % 2 == 0 &&
+         I.bc.src_mode == AMLBM_SRC_LOCAL && (odd || I.Nz % 2 == 0) &&
          9LL * pitch_of(I.Nz) * I.Nr < (1LL << 31);
 }
-bool all_pair_ok(const std::vector<amlbm_instance>& inst) {
+bool all_pair_ok(const std::vector<amlbm_instance>& inst, bool odd = false) {
   for (const auto& I : inst)
-    if (!pair_ok(I)) return false;
+    if (!pair_ok(I, odd)) return false;
   return true;
 }
 
@@ -187,7 +188,7 @@ void pick_tile(int storage, const std::vector<amlbm_instance>& inst, int* sched,
       if (count_tiles(inst, t.tz, t.tr) >= t.least) return;
     }
   }
-  if (all_pair_ok(inst)) {
+  if (all_pair_ok(inst, storage == AMLBM_STORE_F32)) {
     *sched = amlbm::SCHED_PAIR;
     *tz = amlbm::kStripWidth;
     *tr = pick_strip(inst);
@@ -268,16 +269,43 @@ struct Layout {
   long long sumN = 0, sumNz = 0;
 };
 
-Layout make_layout(const std::vector<amlbm_instance>& inst, int storage, int tz, int tr, int sched) {
+// Rows of the read-back's strips, of which 12 per SM are resident: the fewest rounds of
+// rows over the batch, and on equal terms the lowest strips (the read-back of a single
+// instance takes as long as one strip).
+int pick_read_rows(const std::vector<amlbm_instance>& inst) {
+  constexpr int kPlaces = 12 * 152;
+  int best = 4, max_rows = 0;
+  double least = 1e300;
+  for (const auto& I : inst) max_rows = std::max(max_rows, I.Nr);
+  for (int h = 4; h <= 1024; h += h < 128 ? 4 : 32) {
+    long long strips = 0;
+    for (const auto& I : inst)
+      strips += (long long)amlbm::tiles_along_z(amlbm::SCHED_PAIR, amlbm::kStripReadWidth, I.Nz) * ((I.Nr + h - 1) / h);
+    const double rounds = strips > 4 * kPlaces ? (double)strips / kPlaces + 0.5 : (double)((strips + kPlaces - 1) / kPlaces);
+    const double t = rounds * (h + 3.0);
+    if (t < least) {
+      least = t;
+      best = h;
+    }
+    if (h >= max_rows) break;
+  }
+  return best;
+}
+
+// Tile of the read-back kernel.
+void read_tile(const std::vector<amlbm_instance>& inst, int storage, int sched, int tz, int tr, int* rz, int* rr) {
+  amlbm::rb_tile(storage, sched, tz, tr, rz, rr);
+  if (*rz == amlbm::kStripReadWidth) *rr = pick_read_rows(inst);
+}
+
+Layout make_layout(const std::vector<amlbm_instance>& inst, int storage, int tz, int tr, int sched, int rz, int rr) {
   Layout L;
   size_t o = 0;
   auto take = [&](size_t bytes) { const size_t at = o; o = align_up(o + bytes); return at; };
   const size_t n = inst.size();
   for (const auto& I : inst) {
     L.ntiles += amlbm::tiles_along_z(sched, tz, I.Nz) * ((I.Nr + tr - 1) / tr);
-    int rz, rr;
-    amlbm::rb_tile(storage, sched, tz, tr, &rz, &rr);
-    L.rb_ntiles += ((I.Nz + rz - 1) / rz) * ((I.Nr + rr - 1) / rr);
+    L.rb_ntiles += amlbm::tiles_along_z(sched, rz, I.Nz) * ((I.Nr + rr - 1) / rr);
     L.maxN = std::max(L.maxN, I.Nz * I.Nr);
     L.maxNz = std::max(L.maxNz, I.Nz);
     L.diag_nblk = std::max(L.diag_nblk, amlbm::diag_blocks(I.Nz, I.Nr));
@@ -318,11 +346,13 @@ Layout make_layout(const std::vector<amlbm_instance>& inst, int storage, int tz,
 
 struct amlbm_batch {
   int n = 0, storage = 0, sched = 0, tz = 0, tr = 0, graph_chunk = 0;
+  int rz = 0, rr = 0;  // tile of the read-back
   cudaStream_t stream = nullptr;
   char* arena = nullptr;
   size_t arena_bytes = 0;
   bool owns = false;
-  int form = -1;  // launch_step_strip
+  int form = -1;      // launch_step_strip
+  bool odd = false;
   Layout L;
   std::vector<InstDesc> desc;
   std::vector<long long> steps;  // per instance, since its fields were set
@@ -347,7 +377,7 @@ namespace {
 
 int launch_steps_direct(amlbm_batch* b, int n) {
   for (int s = 0; s < n; ++s) {
-    const cudaError_t e = amlbm::launch_step(b->storage, b->sched, b->form, b->tz, b->tr, b->d_desc, b->d_tiles,
+    const cudaError_t e = amlbm::launch_step(b->storage, b->sched, b->form, b->odd, b->tz, b->tr, b->d_desc, b->d_tiles,
                                              b->L.ntiles, 0, b->parity, b->stream, b->d_ctr);
     if (e != cudaSuccess) return fail(AMLBM_ECUDA, std::string("step kernel: ") + cudaGetErrorString(e));
     b->parity ^= 1;
@@ -362,7 +392,7 @@ int ensure_graph(amlbm_batch* b, int parity) {
   int p = parity;
   cudaError_t e = cudaSuccess;
   for (int s = 0; s < b->graph_chunk && e == cudaSuccess; ++s) {
-    e = amlbm::launch_step(b->storage, b->sched, b->form, b->tz, b->tr, b->d_desc, b->d_tiles, b->L.ntiles, 0, p,
+    e = amlbm::launch_step(b->storage, b->sched, b->form, b->odd, b->tz, b->tr, b->d_desc, b->d_tiles, b->L.ntiles, 0, p,
                            b->stream, b->d_ctr);
     p ^= 1;
   }
@@ -428,7 +458,11 @@ int batch_build(const std::vector<amlbm_instance>& inst, const amlbm_tune* tune,
   if (b->graph_chunk % 2) b->graph_chunk += 1;  // even: a chunk returns to its parity
   b->stream = static_cast<cudaStream_t>(stream);
   if (!b->stream) b->graph_chunk = 0;  // the legacy stream cannot be captured
-  b->L = make_layout(inst, storage, tz, tr, sched);
+  int rz, rr;
+  read_tile(inst, storage, sched, tz, tr, &rz, &rr);
+  b->rz = rz;
+  b->rr = rr;
+  b->L = make_layout(inst, storage, tz, tr, sched, rz, rr);
   if (workspace) {
     if (ws_bytes < b->L.total || (reinterpret_cast<uintptr_t>(workspace) % kAlign)) {
       delete b;
@@ -473,13 +507,12 @@ int batch_build(const std::vector<amlbm_instance>& inst, const amlbm_tune* tune,
                : I.bc.rounding == AMLBM_ROUND_STOCHASTIC ? 1
                : I.bc.rounding == AMLBM_ROUND_NEAREST ? 0 : (sr_default ? 1 : 0);
     const int form = plain && d.rounding == (sr_default ? 1 : 0) ? d.shift : -1;
+    b->odd = b->odd || I.Nz % 2 != 0;
     b->form = i == 0 || form == b->form ? form : -1;
     d.tiles_z = amlbm::tiles_along_z(sched, tz, I.Nz);
     d.tiles_r = (I.Nr + tr - 1) / tr;
     d.tile_base = (int)tiles.size();
-    int rz, rr;
-    amlbm::rb_tile(storage, sched, tz, tr, &rz, &rr);
-    d.rb_tiles_z = (I.Nz + rz - 1) / rz;
+    d.rb_tiles_z = amlbm::tiles_along_z(sched, rz, I.Nz);
     d.rb_tiles_r = (I.Nr + rr - 1) / rr;
     d.rb_tile_base = (int)rb_tiles.size();
     d.tau = I.tau;
@@ -547,12 +580,13 @@ int batch_build(const std::vector<amlbm_instance>& inst, const amlbm_tune* tune,
   }
   // the allocation-free diagnostics' scratch: looked up now, in a call that
   // allocates anyway (its failure surfaces at that entry point, not here)
-  int rz, rr;
-  amlbm::rb_tile(storage, sched, tz, tr, &rz, &rr);
   amlbm::noalloc_prepare(storage, rz, rr);
   // the pair read-back's code, loaded now for the same reason (its first use
   // may be an allocation-free diagnostics call)
-  if (sched == amlbm::SCHED_PAIR) amlbm::readback_pair_preload(storage, rz, rr);
+  if (sched == amlbm::SCHED_PAIR) {
+    if (tz == amlbm::kStripWidth) amlbm::readback_strip_preload(storage, b->form, b->odd);
+    else amlbm::readback_pair_preload(storage, rz, rr);
+  }
   *out = b;
   return AMLBM_OK;
 }
@@ -611,8 +645,10 @@ int set_inlet(amlbm_batch* b, int k, const double* uz, const double* ur) {
 
 // rho and u of nt tiles of the read-back list from toff into the read-back planes
 cudaError_t launch_readback(amlbm_batch* b, int nt, int toff) {
-  int rz, rr;
-  amlbm::rb_tile(b->storage, b->sched, b->tz, b->tr, &rz, &rr);
+  const int rz = b->rz, rr = b->rr;
+  if (b->sched == amlbm::SCHED_PAIR && b->tz == amlbm::kStripWidth)
+    return amlbm::launch_readback_strip(b->storage, b->form, b->odd, rr, b->d_desc, b->d_rb_tiles, nt, toff, b->parity,
+                                        b->stream);
   if (b->sched == amlbm::SCHED_PAIR)
     return amlbm::launch_readback_pair(b->storage, rz, rr, b->d_desc, b->d_rb_tiles, nt, toff, b->parity, b->stream);
   return amlbm::launch_macro(b->storage, rz, rr, b->d_desc, b->d_rb_tiles, nt, toff, b->parity, b->stream);
@@ -831,8 +867,12 @@ size_t amlbm_batch_workspace_bytes(int n, const amlbm_instance* inst) {
   for (int sc = amlbm::SCHED_FUSED; sc <= amlbm::SCHED_PAIR; ++sc) {
     int tz[32], tr[32];
     const int nt = std::min(32, amlbm::tile_list(v[0].bc.storage, sc, tz, tr, 32));
-    for (int c = 0; c < nt; ++c)
-      need = std::max(need, make_layout(v, v[0].bc.storage, tz[c], tr[c], sc).total);
+    for (int c = 0; c < nt; ++c) {
+      int rz, rr;
+      amlbm::rb_tile(v[0].bc.storage, sc, tz[c], tr[c], &rz, &rr);
+      if (rz == amlbm::kStripReadWidth) rr = 4;  // the most tiles a read-back may have
+      need = std::max(need, make_layout(v, v[0].bc.storage, tz[c], tr[c], sc, rz, rr).total);
+    }
   }
   return need;
 }

@@ -62,7 +62,7 @@ enum { SCHED_FUSED = 1, SCHED_SPLIT = 2, SCHED_PAIR = 3 };
 // ctr (four ints, zero at creation): tile counters of the persistent fused
 // grid and the step numbers for stochastic rounding, one per parity; nullptr
 // launches one CTA per tile.
-cudaError_t launch_step(int storage, int schedule, int form, int tz, int tr, const InstDesc* d_desc,
+cudaError_t launch_step(int storage, int schedule, int form, bool odd, int tz, int tr, const InstDesc* d_desc,
                         const int* d_tile_inst, int ntiles, int toff, int parity, cudaStream_t s,
                         int* ctr);
 cudaError_t launch_macro(int storage, int tz, int tr, const InstDesc* d_desc,
@@ -70,28 +70,29 @@ cudaError_t launch_macro(int storage, int tz, int tr, const InstDesc* d_desc,
 // Loads the code of the read-back kernel of a storage form on the current
 // device (the CUDA runtime otherwise loads it at its first launch).
 cudaError_t macro_preload(int storage, int rz, int rr);
-// Columns of a strip (amlbm_step_strip.cu); a lattice of at most 64 columns is one strip.
-constexpr int kStripWidth = 48;
+// Columns of a strip (amlbm_step_strip.cu); an even lattice of at most 64 columns is one strip.
+constexpr int kStripWidth = 48, kStripReadWidth = 56;
 // Rows of a strip that the library chooses among: the kernel runs four rows at a time
 // and two more than the strip has.
 constexpr int kStripMaxRows = 1022;
 inline bool strip_rows_ok(int rows) { return rows >= 2 && rows <= kStripMaxRows && rows % 4 == 2; }
-// Tiles of a lattice along z (tz = kStripWidth on the pair schedule: strips).
+// Tiles of a lattice along z (tz = kStripWidth or kStripReadWidth on the pair schedule:
+// strips).
 inline int tiles_along_z(int sched, int tz, int Nz) {
-  if (sched == SCHED_PAIR && tz == kStripWidth && Nz <= 64) return 1;
+  if (sched == SCHED_PAIR && (tz == kStripWidth || tz == kStripReadWidth) && Nz <= 64 && Nz % 2 == 0) return 1;
   return (Nz + tz - 1) / tz;
 }
 
 // Tile of the read-back kernel of a batch whose step runs (sched, tz, tr): the step's
-// own tile on the pair schedule (64 x 16 for strips) and for FP64 on the split one
-// (whose force kernel reads back), else 26 x 16 for the FP32-arithmetic forms (less halo work per site
+// own tile on the pair schedule (strips: 56 columns) and for FP64 on the split one (whose
+// force kernel reads back), else 26 x 16 for the FP32-arithmetic forms (less halo work per site
 // than 32 x 8) and 32 x 8 for FP64.
 inline void rb_tile(int storage, int sched, int tz, int tr, int* rz, int* rr) {
   const bool f64 = storage == 0;  // AMLBM_STORE_F64
   const bool step = sched == SCHED_PAIR || (f64 && sched == SCHED_SPLIT);
   const bool strip = sched == SCHED_PAIR && tz == kStripWidth;
-  *rz = strip ? 64 : step ? tz : f64 ? 32 : 26;
-  *rr = strip ? 16 : step ? tr : f64 ? 8 : 16;
+  *rz = strip ? kStripReadWidth : step ? tz : f64 ? 32 : 26;
+  *rr = step ? tr : f64 ? 8 : 16;  // strips: pick_read_rows (amlbm_abi.cu)
 }
 cudaError_t launch_init(int storage, const InstDesc* d_desc, int inst, int Nz, int Nr,
                         const double* rho, const double* uz, const double* ur, int parity,
@@ -165,10 +166,14 @@ bool pair_tile_supported(int storage, int tz, int tr);
 int pair_tile_list(int storage, int* tz, int* tr, int cap);
 // The strip kernel of the pair schedule (amlbm_step_strip.cu): strips of H rows.  form:
 // the common shift code of lattices that are all axisymmetric with the velocity shift
-// and the storage form's default rounding, or -1.
-cudaError_t launch_step_strip(int storage, int form, int H, const InstDesc* d_desc, const int* d_tile_inst, int ntiles,
-                              int parity, cudaStream_t s, int* ctr);
-cudaError_t launch_step_pair(int storage, int form, int tz, int tr, const InstDesc* d_desc,
+// and the storage form's default rounding, or -1.  odd: there are lattices of odd width
+// (FP32 storage only).  And the read-back of such a batch, with the loading of its code.
+cudaError_t launch_step_strip(int storage, int form, bool odd, int H, const InstDesc* d_desc, const int* d_tile_inst,
+                              int ntiles, int parity, cudaStream_t s, int* ctr);
+cudaError_t launch_readback_strip(int storage, int form, bool odd, int H, const InstDesc* d_desc,
+                                  const int* d_tile_inst, int nt, int toff, int parity, cudaStream_t s);
+cudaError_t readback_strip_preload(int storage, int form, bool odd);
+cudaError_t launch_step_pair(int storage, int form, bool odd, int tz, int tr, const InstDesc* d_desc,
                              const int* d_tile_inst, int ntiles, int parity, cudaStream_t s, int* ctr);
 // The read-back (rho, u into the read-back planes) of a pair batch, whose
 // read-back list is tiled like its step: nt tiles from toff.  And the loading of

@@ -941,11 +941,11 @@ int tile_list(int storage, int sched, int* tz, int* tr, int cap) {
   return n;
 }
 
-cudaError_t launch_step(int storage, int sched, int form, int tz, int tr, const InstDesc* d, const int* ti,
+cudaError_t launch_step(int storage, int sched, int form, bool odd, int tz, int tr, const InstDesc* d, const int* ti,
                         int nt, int toff, int parity, cudaStream_t s, int* ctr) {
   if (sched == SCHED_PAIR) {
     if (toff != 0) return cudaErrorInvalidValue;
-    return launch_step_pair(storage, form, tz, tr, d, ti, nt, parity, s, ctr);
+    return launch_step_pair(storage, form, odd, tz, tr, d, ti, nt, parity, s, ctr);
   }
   if (sched == SCHED_SPLIT && storage == AMLBM_STORE_F64) {
     if (toff != 0) return cudaErrorInvalidValue;

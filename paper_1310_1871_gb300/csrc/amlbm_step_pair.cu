@@ -628,9 +628,9 @@ static cudaError_t pair_kind(int kind, int storage, int tz, int tr, const InstDe
   }
 }
 
-cudaError_t launch_step_pair(int storage, int form, int tz, int tr, const InstDesc* d, const int* ti, int nt, int parity,
+cudaError_t launch_step_pair(int storage, int form, bool odd, int tz, int tr, const InstDesc* d, const int* ti, int nt, int parity,
                              cudaStream_t s, int* ctr) {
-  if (storage != AMLBM_STORE_F64 && tz == kStripWidth) return launch_step_strip(storage, form, tr, d, ti, nt, parity, s, ctr);
+  if (storage != AMLBM_STORE_F64 && tz == kStripWidth) return launch_step_strip(storage, form, odd, tr, d, ti, nt, parity, s, ctr);
   return pair_kind(0, storage, tz, tr, d, ti, nt, 0, parity, s, ctr);
 }
 

@@ -27,7 +27,9 @@
 // Measured (GB300, FP32 storage, us per step; the 64 x 24 tile kernel before): the 64-drop
 // sweep of 835,240 sites 37.7 -> 21.5, eight threads of 3.6 M sites 119.7 -> 64.1,
 // 8192 x 4096 995 -> 521 (80 B per site: 76 % of the measured HBM bandwidth),
-// 256 x 128 9.5 (fused 32 x 8) -> 7.6.
+// 256 x 128 9.5 (fused 32 x 8) -> 7.6, 255 x 65 10.3 (fused) -> 8.1.
+// Read-back (the chain up to the velocity, 12 warps per SM): 8192 x 4096 diagnostics 675 ->
+// 538 us, the sweep's 57 -> 48 (pair tiles of 64 x 16 before).
 //
 // The operations on a site's values are those of the other schedules, in their order, so
 // the states are bit-identical.
@@ -119,15 +121,38 @@ __device__ __forceinline__ F2 take_pair(uint32_t src) {  // a pair of population
     }
   }
 }
-template <class S>
+// A pair of a row: at columns k and k + 1, or with ODD one site at a time, at k and k2 (a
+// lattice of odd width has pairs across its seam, and rows that start off the pairs).
+template <bool ODD, class S>
+__device__ __forceinline__ void copy_pair(uint32_t dst, const S* __restrict__ row, int k, int k2) {
+  if constexpr (ODD) {
+    static_assert(sizeof(S) == 4, "asynchronous copies are at least four bytes");
+    copy_in<4>(dst, row + k);
+    copy_in<4>(dst + 4, row + k2);
+  } else {
+    copy_in<2 * (int)sizeof(S)>(dst, row + k);
+  }
+}
+template <class S, bool ODD>
 __device__ __forceinline__ void copy_pops(uint32_t slot, const S* __restrict__ f, const float* __restrict__ psi,
-                                          int plane, int o, int shift, int lane) {
+                                          int plane, int o, int k, int k2, int shift, int lane) {
   using Q = Flight<S>;
 #pragma unroll
-  for (int i = 0; i < 9; ++i) copy_in<Q::kPair>(slot + Q::kPops + (i * 32 + lane) * Q::kPair, f + (size_t)i * plane + o);
+  for (int i = 0; i < 9; ++i)
+    copy_pair<ODD>(slot + Q::kPops + (i * 32 + lane) * Q::kPair, f + (size_t)i * plane + o, k, k2);
   if (shift == 3) {
-    copy_in<8>(slot + Q::kVel + lane * 8, psi + (size_t)plane + o);
-    copy_in<8>(slot + Q::kVel + (32 + lane) * 8, psi + (size_t)2 * plane + o);
+    copy_pair<ODD>(slot + Q::kVel + lane * 8, psi + (size_t)plane + o, k, k2);
+    copy_pair<ODD>(slot + Q::kVel + (32 + lane) * 8, psi + (size_t)2 * plane + o, k, k2);
+  }
+}
+// The pair's values to p and p + 1; with ODD the second only if the lattice has it.
+template <bool ODD, class S>
+__device__ __forceinline__ void store2(S* p, S a, S b, bool second) {
+  if constexpr (ODD) {
+    p[0] = a;
+    if (second) p[1] = b;
+  } else {
+    st2<S>(p, a, b);
   }
 }
 
@@ -154,10 +179,10 @@ __device__ __forceinline__ void decode_pair(uint32_t slot, int lane, int shift, 
 }
 
 // encode_values on a pair, and the store
-template <class S>
+template <class S, bool ODD>
 __device__ __forceinline__ void store_pair(int shift, const F2* fn, F2 rho, F2 psi, float inv_rho0, float rho0,
                                            float rref, int rounding, uint32_t site, uint32_t step, S* __restrict__ f,
-                                           float* __restrict__ ps, int plane, int o) {
+                                           float* __restrict__ ps, int plane, int o, bool second) {
   float pa, pb;
   unpack(psi, pa, pb);
   F2 base[9];
@@ -172,8 +197,8 @@ __device__ __forceinline__ void store_pair(int shift, const F2* fn, F2 rho, F2 p
       equilibrium(s, vz, vr, fe);
 #pragma unroll
       for (int i = 0; i < 9; ++i) base[i] = fn[i] - fe[i];
-      st2<float>(ps + (size_t)plane + o, lo(vz), hi(vz));
-      st2<float>(ps + (size_t)2 * plane + o, lo(vr), hi(vr));
+      store2<ODD>(ps + (size_t)plane + o, lo(vz), hi(vz), second);
+      store2<ODD>(ps + (size_t)2 * plane + o, lo(vr), hi(vr), second);
     } else {
 #pragma unroll
       for (int i = 0; i < 9; ++i) base[i] = fma(lit<F2>(-w_(i)), s, fn[i]);
@@ -203,31 +228,37 @@ __device__ __forceinline__ void store_pair(int shift, const F2* fn, F2 rho, F2 p
       *reinterpret_cast<__nv_bfloat162*>(out) = __floats2bfloat162_rn(a, b);
     } else {
       unpack(base[i], a, b);
-      st2<S>(out, a, b);
+      store2<ODD>(out, a, b, second);
     }
   }
-  st2<float>(ps + o, pa, pb);
+  store2<ODD>(ps + o, pa, pb, second);
 }
 
 // One strip.  FORM: the shift code of a batch whose lattices are all axisymmetric with
 // the velocity shift and the storage form's default rounding, so that nothing in the
 // marching loop branches on the lattice's options; or kAnyForm.
+// ODD: lattices of odd width among them (FP32 storage).  READ: no step, but rho and u of
+// the strip's rows into the read-back planes: the chain up to the velocity, which
+// reaches 4 sites, so the strip is 56 columns wide and starts 4 rows early.
 constexpr int kAnyForm = -1;
-template <class S, int FORM>
+template <class S, int FORM, bool ODD, bool READ>
 __device__ __forceinline__ void march(const InstDesc& D, int tile, int H, int parity, int* __restrict__ ctr,
-                                      F2* __restrict__ ring,
-                                      uint32_t flight) {
+                                      F2* __restrict__ ring, uint32_t flight) {
+  constexpr int kHalo = READ ? 4 : 8, kWidth = 64 - 2 * kHalo, kEarly = READ ? 4 : 7;
+  static_assert(READ ? kWidth == kStripReadWidth : kWidth == kStripWidth, "the tiling of the host");
   const int lane = threadIdx.x;
   const int Nz = D.Nz, Nr = D.Nr, P = D.P, plane = P * Nr;
-  const int l = tile - D.tile_base;
-  const bool whole = Nz <= 64;  // the strip is the whole period
+  const int l = tile - (READ ? D.rb_tile_base : D.tile_base), tz = READ ? D.rb_tiles_z : D.tiles_z;
+  const bool whole = Nz <= 64 && (!ODD || Nz % 2 == 0);  // the strip is the whole period
   const int n = Nz >> 1;
-  const int j0 = (l / D.tiles_z) * H, j1 = min(j0 + H, Nr);
-  const int col = whole ? 2 * lane : (l % D.tiles_z) * kStripWidth - 8 + 2 * lane;
-  const int kk = whole ? (col < Nz ? col : 0) : (col < 0 ? col + Nz : (col >= Nz ? col - Nz : col));
+  const int j0 = (l / tz) * H, j1 = min(j0 + H, Nr);
+  const int col = whole ? 2 * lane : (l % tz) * kWidth - kHalo + 2 * lane;
+  const int kk = ODD ? wrapz(col, Nz)
+                     : whole ? (col < Nz ? col : 0) : (col < 0 ? col + Nz : (col >= Nz ? col - Nz : col));
+  const int k2 = ODD ? wrapz(col + 1, Nz) : kk + 1;
   const int left = whole && lane == 0 ? n - 1 : (lane + 31) & 31;
   const int right = whole && lane == n - 1 ? 0 : (lane + 1) & 31;
-  const bool mine = (whole || (lane >= 4 && lane < 28)) && col < Nz;
+  const bool mine = (whole || (lane >= kHalo / 2 && lane < 32 - kHalo / 2)) && col < Nz, second = col + 1 < Nz;
   const S* __restrict__ fin = static_cast<const S*>(D.f[parity]);
   const float* __restrict__ psin = static_cast<const float*>(D.psi[parity]);
   S* __restrict__ fout = static_cast<S*>(D.f[parity ^ 1]);
@@ -267,14 +298,17 @@ __device__ __forceinline__ void march(const InstDesc& D, int tile, int H, int pa
   float nirs = 0.0f;
   using Q = Flight<S>;
   auto copy_psi = [&](int r, int ph) {
-    copy_in<8>(flight + ph * Q::kSlot + Q::kPsi + lane * 8, psin + reflect_row(r, Nr) * P + kk);
+    copy_pair<ODD>(flight + ph * Q::kSlot + Q::kPsi + lane * 8, psin + reflect_row(r, Nr) * P, kk, k2);
   };
   pdl_wait();  // everything above reads only what creation wrote
-  const uint32_t step = (uint32_t)ctr[2 + parity];
-  if (blockIdx.x == 0 && lane == 0) ctr[2 + (parity ^ 1)] = (int)(step + 1);
+  uint32_t step = 0;
+  if constexpr (!READ) {
+    step = (uint32_t)ctr[2 + parity];
+    if (blockIdx.x == 0 && lane == 0) ctr[2 + (parity ^ 1)] = (int)(step + 1);
+  }
 #pragma unroll
   for (int ph = 0; ph < 4; ++ph) {
-    copy_psi(j0 - 7 + ph, ph);
+    copy_psi(j0 - kEarly + ph, ph);
     commit_copies();
   }
 
@@ -290,7 +324,8 @@ __device__ __forceinline__ void march(const InstDesc& D, int tile, int H, int pa
     F2 f[9];
     if constexpr (F_ON) decode_pair<S>(slot, lane, shift, C[PH], inv_rho0, rho0, rref, f);  // row r - 4
     copy_psi(r + 4, PH);
-    if constexpr (F_NEXT) copy_pops<S>(slot, fin, psin, plane, min(max(r, 0), Nr - 1) * P + kk, shift, lane);
+    if constexpr (F_NEXT)
+      copy_pops<S, ODD>(slot, fin, psin, plane, min(max(r, 0), Nr - 1) * P, kk, k2, shift, lane);
     commit_copies();
     const Row5 p = neighbours(pc, left, right);
 
@@ -344,6 +379,15 @@ __device__ __forceinline__ void march(const InstDesc& D, int tile, int H, int pa
       Fz = fma(rho, q.gz, Fz);
       const F2 inv_rho = rcp(rho);
       F2 uz = fma(Fz, lit<F2>(0.5), jz) * inv_rho, ur = fma(Fr, lit<F2>(0.5), jr) * inv_rho;
+      if constexpr (READ) {
+        if (mine && j < j1) {
+          const int w = j * Nz + col;
+          store2<ODD>(static_cast<float*>(D.rho_out) + w, lo(rho), hi(rho), second);
+          store2<ODD>(static_cast<float*>(D.uz_out) + w, lo(uz), hi(uz), second);
+          store2<ODD>(static_cast<float*>(D.ur_out) + w, lo(ur), hi(ur), second);
+        }
+        return;
+      }
       collide(q, guo, gk, f, rho, uz, ur, jz, jr, Fz, Fr, inv_rho,
               [&](int i, F2 v) { ring[(PH * 9 + i) * 32] = v; });
       // Ghost rows of u (depth 2): rows -1, -2 mirror rows 0, 1 about the axis (u_z even,
@@ -394,8 +438,8 @@ __device__ __forceinline__ void march(const InstDesc& D, int tile, int H, int pa
           const F2 rn = moment0(fn);
           const F2 pn = psi_of(q, rn);
           if (mine)
-            store_pair<S>(shift, fn, rn, pn, inv_rho0, rho0, rref, rounding, (uint32_t)(o * Nz + col), step, fout,
-                          psout, plane, o * P + col);
+            store_pair<S, ODD>(shift, fn, rn, pn, inv_rho0, rho0, rref, rounding, (uint32_t)(o * Nz + col), step, fout,
+                                 psout, plane, o * P + col, second);
         }
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
@@ -425,7 +469,7 @@ __device__ __forceinline__ void march(const InstDesc& D, int tile, int H, int pa
   using std::integral_constant;
   using Off = integral_constant<bool, false>;
   using On = integral_constant<bool, true>;
-  int r = j0 - 7;
+  int r = j0 - kEarly;
   auto rows4 = [&](auto F_NEXTc, auto F_ONc, auto S_ONc) {
     row(r, integral_constant<int, 0>(), F_NEXTc, F_ONc, S_ONc);
     row(r + 1, integral_constant<int, 1>(), F_NEXTc, F_ONc, S_ONc);
@@ -437,54 +481,99 @@ __device__ __forceinline__ void march(const InstDesc& D, int tile, int H, int pa
   rows4(On(), Off(), Off());
   radii(r - 4);
   rows4(On(), On(), Off());
+  using Rest = integral_constant<bool, !READ>;
 #pragma unroll 1
-  while (r < j1 + 7) {
+  while (r < j1 + kEarly) {
     if (r - 4 - jb == 32) radii(r - 4);
-    rows4(On(), On(), On());
+    rows4(On(), On(), Rest());
   }
   asm volatile("cp.async.wait_all;");
 }
 
-template <class S, int FORM>
+template <class S, int FORM, bool ODD>
 __global__ void __launch_bounds__(32, 8) strip_step(const InstDesc* __restrict__ descs,
-                                                                 const int* __restrict__ tile_inst, int H,
-                                                                 int parity, int* __restrict__ ctr) {
+                                                    const int* __restrict__ tile_inst, int H, int parity,
+                                                    int* __restrict__ ctr) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  march<S, FORM>(descs[tile_inst[blockIdx.x]], blockIdx.x, H, parity, ctr, reinterpret_cast<F2*>(smem_raw),
-                 (uint32_t)__cvta_generic_to_shared(smem_raw) + kRingBytes);
+  march<S, FORM, ODD, false>(descs[tile_inst[blockIdx.x]], blockIdx.x, H, parity, ctr,
+                             reinterpret_cast<F2*>(smem_raw),
+                             (uint32_t)__cvta_generic_to_shared(smem_raw) + kRingBytes);
   pdl_trigger();
 }
 
-template <class S, int FORM>
-cudaError_t strip_t(const InstDesc* d, const int* ti, int nt, int H, int parity, cudaStream_t s, int* ctr) {
+template <class S, int FORM, bool ODD>
+__global__ void __launch_bounds__(32, 12) strip_read(const InstDesc* __restrict__ descs,
+                                                     const int* __restrict__ tile_inst, int toff, int H, int parity) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int tile = blockIdx.x + toff;
+  march<S, FORM, ODD, true>(descs[tile_inst[tile]], tile, H, parity, nullptr, nullptr,
+                            (uint32_t)__cvta_generic_to_shared(smem_raw));
+  pdl_trigger();
+}
+
+// What to launch: a step or a read-back of nt tiles from toff, or the loading of the
+// read-back's code.
+struct Call {
+  enum { kStep, kRead, kLoad } kind;
+  int form, H, nt, toff, parity;
+  bool odd;
+  const InstDesc* d;
+  const int* ti;
+  cudaStream_t s;
+  int* ctr;
+};
+
+template <class S, int FORM, bool ODD>
+cudaError_t issue(const Call& c) {
   constexpr size_t smem = kRingBytes + Flight<S>::kBytes;
   static_assert(smem <= 48 * 1024, "within the default shared-memory limit");
-  return launch_pdl(strip_step<S, FORM>, nt, 32, smem, s, d, ti, H, parity, ctr);
+  if (c.kind == Call::kStep)
+    return launch_pdl(strip_step<S, FORM, ODD>, c.nt, 32, smem, c.s, c.d, c.ti, c.H, c.parity, c.ctr);
+  // the read-back branches on the shift of the 16-bit forms
+  constexpr int F = sizeof(S) == 4 ? FORM : kAnyForm;
+  if (c.kind == Call::kRead)
+    return launch_pdl(strip_read<S, F, ODD>, c.nt, 32, (size_t)Flight<S>::kBytes, c.s, c.d, c.ti, c.toff, c.H,
+                      c.parity);
+  cudaFuncAttributes a;
+  return cudaFuncGetAttributes(&a, strip_read<S, F, ODD>);
+}
+
+cudaError_t choose(int storage, const Call& c) {
+  if (c.odd) {
+    if (storage != AMLBM_STORE_F32) return cudaErrorInvalidValue;
+    return c.form == 0 ? issue<float, 0, true>(c) : issue<float, kAnyForm, true>(c);
+  }
+  switch (storage) {
+    case AMLBM_STORE_F32: return c.form == 0 ? issue<float, 0, false>(c) : issue<float, kAnyForm, false>(c);
+    case AMLBM_STORE_F16:
+      return c.form == 2   ? issue<__half, 2, false>(c)
+             : c.form == 3 ? issue<__half, 3, false>(c)
+                           : issue<__half, kAnyForm, false>(c);
+    case AMLBM_STORE_BF16:
+      return c.form == 2   ? issue<__nv_bfloat16, 2, false>(c)
+             : c.form == 3 ? issue<__nv_bfloat16, 3, false>(c)
+                           : issue<__nv_bfloat16, kAnyForm, false>(c);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 }  // namespace
 
-cudaError_t launch_step_strip(int storage, int form, int H, const InstDesc* d, const int* ti, int nt, int parity, cudaStream_t s,
-                              int* ctr) {
+cudaError_t launch_step_strip(int storage, int form, bool odd, int H, const InstDesc* d, const int* ti, int nt,
+                              int parity, cudaStream_t s, int* ctr) {
   if (nt <= 0) return cudaSuccess;
   if (!ctr) return cudaErrorInvalidValue;
-  switch (storage) {
-#define AMLBM_STRIP(S, F) \
-  if (form == F || F == kAnyForm) return strip_t<S, F>(d, ti, nt, H, parity, s, ctr)
-    case AMLBM_STORE_F32:
-      AMLBM_STRIP(float, 0);
-      AMLBM_STRIP(float, kAnyForm);
-    case AMLBM_STORE_F16:
-      AMLBM_STRIP(__half, 2);
-      AMLBM_STRIP(__half, 3);
-      AMLBM_STRIP(__half, kAnyForm);
-    case AMLBM_STORE_BF16:
-      AMLBM_STRIP(__nv_bfloat16, 2);
-      AMLBM_STRIP(__nv_bfloat16, 3);
-      AMLBM_STRIP(__nv_bfloat16, kAnyForm);
-#undef AMLBM_STRIP
-    default: return cudaErrorInvalidValue;
-  }
+  return choose(storage, {Call::kStep, form, H, nt, 0, parity, odd, d, ti, s, ctr});
+}
+
+cudaError_t launch_readback_strip(int storage, int form, bool odd, int H, const InstDesc* d, const int* ti, int nt,
+                                  int toff, int parity, cudaStream_t s) {
+  if (nt <= 0) return cudaSuccess;
+  return choose(storage, {Call::kRead, form, H, nt, toff, parity, odd, d, ti, s, nullptr});
+}
+
+cudaError_t readback_strip_preload(int storage, int form, bool odd) {
+  return choose(storage, {Call::kLoad, form, 0, 0, 0, 0, odd, nullptr, nullptr, nullptr, nullptr});
 }
 
 }  // namespace amlbm

@@ -48,6 +48,23 @@ def test_strips_equal_fused_bitwise(Nz, Nr, storage, kw):
             assert np.array_equal(a, b), (kind, np.abs(a - b).max())
 
 
+@pytest.mark.parametrize("kw", [dict(), dict(wall="noslip", gz=1e-4, forcing="guo"), dict(shift="equilibrium"),
+                                dict(axisym=False)])
+@pytest.mark.parametrize("Nz,Nr", [(1, 8), (3, 5), (47, 9), (49, 4), (63, 33), (65, 20), (97, 61), (255, 65)])
+def test_odd_widths_equal_fused_bitwise(Nz, Nr, kw):
+    """FP32 lattices of odd width, alone and beside even ones (among them one that is a
+    single strip): the library's own choice; a requested pair schedule refuses them."""
+    odd = amlbm.InstanceSpec(Nz, Nr, 0.9, -4.9, **kw)
+    for specs in ([odd], [amlbm.InstanceSpec(64, 12, 0.9, -4.9), odd, amlbm.InstanceSpec(150, 31, 1.0, -5.0)]):
+        ref, _ = run(specs, "f32", 20, tile=(32, 8), schedule="fused")
+        got, kind = run(specs, "f32", 20)
+        assert kind[0] == "pair" and kind[1][0] == 48
+        for a, b in zip(ref, got):
+            assert np.array_equal(a, b), (kind, np.abs(a - b).max())
+    with pytest.raises(amlbm.AmlbmError):
+        amlbm.Batch([odd], storage="f32", tile=(48, 6), schedule="pair")
+
+
 @pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
 def test_strips_of_mixed_lattices_equal_fused_bitwise(storage):
     """Different sizes, walls, forcings and shifts in one batch (the kernel that branches on
