@@ -9,6 +9,7 @@
 #include <cstdint>
 #include <cstring>
 #include <functional>
+#include <map>
 #include <new>
 #include <string>
 #include <vector>
@@ -129,7 +130,6 @@ int pick_strip(const std::vector<amlbm_instance>& inst) {
   int best = 2, max_rows = 0;
   double least = 1e300;
   for (const auto& I : inst) max_rows = std::max(max_rows, I.Nr);
-  std::vector<double> busy;
   for (int h = 2; h <= amlbm::kStripMaxRows; h += h < 126 ? 4 : 32) {
     long long strips = 0;
     double sum = 0.0, longest = 0.0;
@@ -143,19 +143,24 @@ int pick_strip(const std::vector<amlbm_instance>& inst) {
     double t = longest;
     if (strips > 4 * kPlaces) {
       t = sum / kPlaces + 0.5 * longest;
-    } else if (strips > kPlaces) {  // in the order of the strips
-      busy.assign(kPlaces, 0.0);
-      t = 0.0;
+    } else if (strips > kPlaces) {  // in the order of the strips, the places that end together at once
+      std::map<double, long long> ends{{0.0, kPlaces}};
+      auto take = [&](long long n, double c) {
+        while (n > 0) {
+          const auto first = *ends.begin();
+          const long long m = std::min(n, first.second);
+          ends.erase(ends.begin());
+          if (m < first.second) ends[first.first] = first.second - m;
+          ends[first.first + c] += m;
+          n -= m;
+        }
+      };
       for (const auto& I : inst) {
-        const int nz = amlbm::tiles_along_z(amlbm::SCHED_PAIR, amlbm::kStripWidth, I.Nz);
-        for (int j = 0; j < I.Nr; j += h)
-          for (int z = 0; z < nz; ++z) {
-            std::pop_heap(busy.begin(), busy.end(), std::greater<double>());
-            busy.back() += cost(std::min(h, I.Nr - j));
-            t = std::max(t, busy.back());
-            std::push_heap(busy.begin(), busy.end(), std::greater<double>());
-          }
+        const long long nz = amlbm::tiles_along_z(amlbm::SCHED_PAIR, amlbm::kStripWidth, I.Nz);
+        take(nz * (I.Nr / h), cost(h));
+        if (I.Nr % h) take(nz, cost(I.Nr % h));
       }
+      t = ends.rbegin()->first;
     }
     if (t < least) {
       least = t;
@@ -175,9 +180,10 @@ int pick_strip(const std::vector<amlbm_instance>& inst) {
 // 1024 x 512 338 / 250 / 227 / 218 (before: 394); 330,400 sites in 25 lattices 217 / 168 /
 // 158.5 / 164.5.
 //
-// FP32 arithmetic: the pair schedule's strips where every lattice allows it (pick_strip),
-// else the fused schedule, with the first tile of a preference list that still gives
-// every SM two CTAs over the whole batch.
+// FP32 arithmetic: the row kernel's tiles while they all run at once (row_height), then
+// the pair schedule's strips where every lattice allows them (pick_strip), else the fused
+// schedule: two rounds of the row kernel's largest tiles (512 x 256: 10.5 us per step; the
+// persistent grid on 26 x 16 14.4), beyond that the persistent grid (1024 x 512: 28.7; rows 36).
 void pick_tile(int storage, const std::vector<amlbm_instance>& inst, int* sched, int* tz, int* tr) {
   if (storage == AMLBM_STORE_F64) {
     static const struct { int tz, tr, least; } pref64[] = {{32, 16, 912}, {32, 8, 96}, {16, 8, 128}, {8, 4, 0}};
@@ -188,19 +194,21 @@ void pick_tile(int storage, const std::vector<amlbm_instance>& inst, int* sched,
       if (count_tiles(inst, t.tz, t.tr) >= t.least) return;
     }
   }
+  *sched = amlbm::SCHED_FUSED;
+  *tz = amlbm::kRowWidth;
+  *tr = amlbm::row_height([&](int h) { return count_tiles(inst, amlbm::kRowWidth, h); });
+  if (*tr) return;
   if (all_pair_ok(inst, storage == AMLBM_STORE_F32)) {
     *sched = amlbm::SCHED_PAIR;
     *tz = amlbm::kStripWidth;
     *tr = pick_strip(inst);
     return;
   }
-  static const int pref32[][2] = {{26, 16}, {64, 8}, {32, 8}};
-  *sched = amlbm::SCHED_FUSED;
-  for (const auto& t : pref32) {
-    *tz = t[0];
-    *tr = t[1];
-    if (count_tiles(inst, *tz, *tr) >= 2 * 152) return;
+  if (count_tiles(inst, amlbm::kRowWidth, amlbm::kRowMaxRows) <= 4 * 152) {
+    *tr = amlbm::kRowMaxRows;
+    return;
   }
+  *tr = 16;
 }
 
 // Shift code the kernels use: 0 none, 1 global rho_ref, 2 local (from psi),
@@ -378,7 +386,7 @@ namespace {
 int launch_steps_direct(amlbm_batch* b, int n) {
   for (int s = 0; s < n; ++s) {
     const cudaError_t e = amlbm::launch_step(b->storage, b->sched, b->form, b->odd, b->tz, b->tr, b->d_desc, b->d_tiles,
-                                             b->L.ntiles, 0, b->parity, b->stream, b->d_ctr);
+                                             b->L.ntiles, b->parity, b->stream, b->d_ctr);
     if (e != cudaSuccess) return fail(AMLBM_ECUDA, std::string("step kernel: ") + cudaGetErrorString(e));
     b->parity ^= 1;
   }
@@ -392,7 +400,7 @@ int ensure_graph(amlbm_batch* b, int parity) {
   int p = parity;
   cudaError_t e = cudaSuccess;
   for (int s = 0; s < b->graph_chunk && e == cudaSuccess; ++s) {
-    e = amlbm::launch_step(b->storage, b->sched, b->form, b->odd, b->tz, b->tr, b->d_desc, b->d_tiles, b->L.ntiles, 0, p,
+    e = amlbm::launch_step(b->storage, b->sched, b->form, b->odd, b->tz, b->tr, b->d_desc, b->d_tiles, b->L.ntiles, p,
                            b->stream, b->d_ctr);
     p ^= 1;
   }

@@ -60,16 +60,30 @@ static_assert(K_CMU12 + 1 == kStepConstants, "one slot per constant");
 // adjacent z-sites per thread; amlbm_step_pair.cu).
 enum { SCHED_FUSED = 1, SCHED_SPLIT = 2, SCHED_PAIR = 3 };
 // ctr (four ints, zero at creation): tile counters of the persistent fused
-// grid and the step numbers for stochastic rounding, one per parity; nullptr
-// launches one CTA per tile.
+// grid and the step numbers for stochastic rounding, one per parity.
 cudaError_t launch_step(int storage, int schedule, int form, bool odd, int tz, int tr, const InstDesc* d_desc,
-                        const int* d_tile_inst, int ntiles, int toff, int parity, cudaStream_t s,
-                        int* ctr);
+                        const int* d_tile_inst, int ntiles, int parity, cudaStream_t s, int* ctr);
 cudaError_t launch_macro(int storage, int tz, int tr, const InstDesc* d_desc,
                          const int* d_tile_inst, int ntiles, int toff, int parity, cudaStream_t s);
 // Loads the code of the read-back kernel of a storage form on the current
 // device (the CUDA runtime otherwise loads it at its first launch).
 cudaError_t macro_preload(int storage, int rz, int rr);
+// The row kernel's tiles (amlbm_step_row.cu): kRowWidth x H sites.
+constexpr int kRowWidth = 26, kRowMinRows = 4, kRowMaxRows = 10;
+// Rows of its tiles: the fewest that leave an SM at most one CTA, else at most the two that
+// fit; 0 when that takes more than kRowMaxRows.  tiles(H): the tiles of H rows.  Measured, us
+// per step for H = 4 .. 10: 64 x 32 3.2 3.3 3.4 3.5 3.6 3.7 3.7; 255 x 65 4.0 (170 tiles) 3.6
+// 3.7 3.8 3.9 3.8 3.8; 256 x 128 4.8 4.2 4.2 4.6 4.8 (160) 4.1 4.1; 512 x 128 8.7 8.4 7.6 7.9
+// 8.0 (320) 5.2 (300) 5.3.  The strips take 7.2, 8.2, 7.7 and 7.7 there; on 512 x 256, which
+// has 520 tiles of 10 rows, 10.0 against 10.5.
+template <class F>
+inline int row_height(F&& tiles) {
+  for (const int most : {152, 2 * 152})
+    for (int H = 4; H <= 10; ++H)
+      if (tiles(H) <= most) return H;
+  return 0;
+}
+inline bool row_rows_ok(int H) { return H >= kRowMinRows && H <= kRowMaxRows; }
 // Columns of a strip (amlbm_step_strip.cu); an even lattice of at most 64 columns is one strip.
 constexpr int kStripWidth = 48, kStripReadWidth = 56;
 // Rows of a strip that the library chooses among: the kernel runs four rows at a time
@@ -85,14 +99,13 @@ inline int tiles_along_z(int sched, int tz, int Nz) {
 
 // Tile of the read-back kernel of a batch whose step runs (sched, tz, tr): the step's
 // own tile on the pair schedule (strips: 56 columns) and for FP64 on the split one (whose
-// force kernel reads back), else 26 x 16 for the FP32-arithmetic forms (less halo work per site
-// than 32 x 8) and 32 x 8 for FP64.
+// force kernel reads back), else 32 x 8 (FP32-arithmetic forms: the row kernel's).
 inline void rb_tile(int storage, int sched, int tz, int tr, int* rz, int* rr) {
   const bool f64 = storage == 0;  // AMLBM_STORE_F64
   const bool step = sched == SCHED_PAIR || (f64 && sched == SCHED_SPLIT);
   const bool strip = sched == SCHED_PAIR && tz == kStripWidth;
-  *rz = strip ? kStripReadWidth : step ? tz : f64 ? 32 : 26;
-  *rr = step ? tr : f64 ? 8 : 16;  // strips: pick_read_rows (amlbm_abi.cu)
+  *rz = strip ? kStripReadWidth : step ? tz : 32;
+  *rr = step ? tr : 8;  // strips: pick_read_rows (amlbm_abi.cu)
 }
 cudaError_t launch_init(int storage, const InstDesc* d_desc, int inst, int Nz, int Nr,
                         const double* rho, const double* uz, const double* ur, int parity,
@@ -113,11 +126,18 @@ enum InterField {
 // inter_tile() is its tile; fstar: 9 scratch planes of the FP64 form (else unused).
 cudaError_t launch_step_inter(int storage, int tz, int tr, const InstDesc* d_desc, const int* d_tile_inst,
                               int ntiles, void* inter, size_t plane, void* fstar, cudaStream_t s);
-// FP64: 8 x 4 where 32 x 8 would leave too many SMs without a tile (pick_tile).
+// FP64: 8 x 4 where 32 x 8 would leave too many SMs without a tile (pick_tile).  FP32: the
+// row kernel's tiles.
 inline void inter_tile(int storage, int Nz, int Nr, int* tz, int* tr) {
-  const bool small = storage == 0 && ((Nz + 31) / 32) * ((Nr + 7) / 8) < 96;  // AMLBM_STORE_F64
-  *tz = small ? 8 : 32;
-  *tr = small ? 4 : 8;
+  if (storage == 0) {  // AMLBM_STORE_F64
+    const bool small = ((Nz + 31) / 32) * ((Nr + 7) / 8) < 96;
+    *tz = small ? 8 : 32;
+    *tr = small ? 4 : 8;
+    return;
+  }
+  const int H = row_height([&](int h) { return (long long)((Nz + kRowWidth - 1) / kRowWidth) * ((Nr + h - 1) / h); });
+  *tz = kRowWidth;
+  *tr = H ? H : kRowMaxRows;
 }
 // Diagnostics (amlbm_diag.cu) of the state whose rho / u the read-back kernel
 // has written: partial sums into `partials` (nblk x 8 doubles) and the Nz column
@@ -173,6 +193,16 @@ cudaError_t launch_step_strip(int storage, int form, bool odd, int H, const Inst
 cudaError_t launch_readback_strip(int storage, int form, bool odd, int H, const InstDesc* d_desc,
                                   const int* d_tile_inst, int nt, int toff, int parity, cudaStream_t s);
 cudaError_t readback_strip_preload(int storage, int form, bool odd);
+// The row kernel (amlbm_step_row.cu): the fused schedule's tiles of kRowWidth x H sites for
+// the FP32-arithmetic forms, any lattice; the read-back of every batch of those forms on
+// the fused or split schedule; and launch_step_inter of FP32 storage.
+cudaError_t launch_step_row(int storage, int H, const InstDesc* d_desc, const int* d_tile_inst, int ntiles, int parity,
+                            cudaStream_t s, int* ctr);
+cudaError_t launch_readback_row(int storage, const InstDesc* d_desc, const int* d_tile_inst, int nt, int toff,
+                                int parity, cudaStream_t s);
+cudaError_t readback_row_preload(int storage);
+cudaError_t launch_step_inter_row(int H, const InstDesc* d_desc, const int* d_tile_inst, int ntiles, float* inter,
+                                  size_t iplane, cudaStream_t s);
 cudaError_t launch_step_pair(int storage, int form, bool odd, int tz, int tr, const InstDesc* d_desc,
                              const int* d_tile_inst, int ntiles, int parity, cudaStream_t s, int* ctr);
 // The read-back (rho, u into the read-back planes) of a pair batch, whose

@@ -83,13 +83,10 @@ struct Tile {
   int inst, k0, j0;
 };
 
-__device__ __forceinline__ Tile tile_of(const InstDesc* descs, const int* tile_inst, int b, int BZ,
-                                        int BR, bool readback = false) {
+__device__ __forceinline__ Tile tile_of(const InstDesc* descs, const int* tile_inst, int b, int BZ, int BR) {
   Tile t;
   t.inst = tile_inst[b];
-  const int tb = readback ? descs[t.inst].rb_tile_base : descs[t.inst].tile_base;
-  const int tz = readback ? descs[t.inst].rb_tiles_z : descs[t.inst].tiles_z;
-  const int l = b - tb;
+  const int tz = descs[t.inst].tiles_z, l = b - descs[t.inst].tile_base;
   t.k0 = (l % tz) * BZ;
   t.j0 = (l / tz) * BR;
   return t;
@@ -107,15 +104,9 @@ struct MinBlocks {
 };
 
 // The fused update of one BZ x BR tile in the lane type T of the storage form.
-// MODE 0: the timestep; MODE 1 (read-back): only rho and u of the tile; MODE 3:
-// the timestep and the forward intermediates of the state it starts from, for
-// the adjoint (into `inter`, I_COUNT planes of `iplane` elements).
-template <class S, class T, int BZ, int BR, int MODE>
-__device__ __forceinline__ void lbm_tile(const InstDesc* __restrict__ descs,
-                                         const int* __restrict__ tile_inst, int tile, int parity,
-                                         typename Store<S>::C* __restrict__ inter, size_t iplane,
-                                         uint32_t step = 0) {
-  constexpr bool READBACK = MODE == 1;
+template <class S, class T, int BZ, int BR>
+__device__ __forceinline__ void lbm_tile(const InstDesc* __restrict__ descs, const int* __restrict__ tile_inst,
+                                         int tile, int parity, uint32_t step) {
   using C = typename Store<S>::C;
   using G = Geo<T, BZ, BR>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -132,7 +123,7 @@ __device__ __forceinline__ void lbm_tile(const InstDesc* __restrict__ descs,
   T* sUr = sUz + G::nF;
   T* sFs = sUr + G::nF;
 
-  const Tile Tl = tile_of(descs, tile_inst, tile, BZ, BR, READBACK);
+  const Tile Tl = tile_of(descs, tile_inst, tile, BZ, BR);
   const InstDesc& D = descs[Tl.inst];
   const int Nz = D.Nz, Nr = D.Nr, P = D.P, k0 = Tl.k0, j0 = Tl.j0;
   const size_t plane = (size_t)P * Nr;
@@ -204,44 +195,13 @@ __device__ __forceinline__ void lbm_tile(const InstDesc* __restrict__ descs,
     sRho[fi] = rho;
     sUz[fi] = uz;
     sUr[fi] = ur;
-    if constexpr (MODE == 3) {
-      if (lr >= G::HF && lr < G::HF + BR && lc >= G::HF && lc < G::HF + BZ && k0 + lc - G::HF < Nz) {
-        C* o = inter + (size_t)j * P + (k0 + lc - G::HF);
-        o[I_RHO * iplane] = (rho).v;
-        o[I_UZ * iplane] = (uz).v;
-        o[I_UR * iplane] = (ur).v;
-        o[I_VZ * iplane] = (fma(Fz, q.tau, jz) * inv_rho).v;
-        o[I_VR * iplane] = (fma(Fr, q.tau, jr) * inv_rho).v;
-        o[I_FZ * iplane] = (Fz).v;
-        o[I_FR * iplane] = (Fr).v;
-        o[I_PSI * iplane] = (psi).v;
-        o[I_SZ * iplane] = unscale(sz, 36.0).v;
-        o[I_SR * iplane] = unscale(sr, 36.0).v;
-        o[I_DR * iplane] = unscale(dr0, 36.0).v;
-        o[I_DRR * iplane] = unscale(Drr, 1296.0).v;
-        o[I_DZR * iplane] = unscale(Dzr, 144.0).v;
-      }
-    }
-    if ((MODE == 0 || MODE == 3) && srow && lc >= 2 && lc < G::FZ - 2) {
+    if (srow && lc >= 2 && lc < G::FZ - 2) {
       T* out = sFs + (lr - 2) * G::SZ + (lc - 2);
       collide(q, guo, splat<T>(kc(D, K_GUO, C())), f, rho, uz, ur, jz, jr, Fz, Fr, inv_rho,
               [&](int i, T v) { out[i * G::nS] = v; });
     }
   });
   __syncthreads();
-
-  if constexpr (READBACK) {
-    for_tile<BR, BZ>([&](int lr, int lc) {
-      const int j = j0 + lr, k = k0 + lc;
-      if (j >= Nr || k >= Nz) return;
-      const int fi = (lr + G::HF) * G::FZ + (lc + G::HF);
-      const size_t o = (size_t)j * Nz + k;
-      static_cast<C*>(D.rho_out)[o] = (sRho[fi]).v;
-      static_cast<C*>(D.uz_out)[o] = (sUz[fi]).v;
-      static_cast<C*>(D.ur_out)[o] = (sUr[fi]).v;
-    });
-    return;
-  }
 
   // Ghost columns of u (depth 2) at the z walls: u_z and u_r odd (no-slip) about
   // the wall half a spacing beyond the first and last columns.
@@ -337,14 +297,6 @@ __device__ __forceinline__ void lbm_tile(const InstDesc* __restrict__ descs,
       const T druz = d1(sUz + fi, G::FZ);
       const T dzur = d1(sUr + fi, 1);
       const T drur = d1(sUr + fi, G::FZ);
-      if constexpr (MODE == 3) {
-        if (lr >= 1 && lr <= BR && lc >= 1 && lc <= BZ && k0 + lc - 1 < Nz) {
-          C* o = inter + (size_t)j * P + (k0 + lc - 1);
-          o[I_G1 * iplane] = unscale(druz, 12.0).v;
-          o[I_G2 * iplane] = unscale(dzur, 12.0).v;
-          o[I_G3 * iplane] = unscale(drur, 12.0).v;
-        }
-      }
       site_sources(q, sRho[fi], sUz[fi], sUr[fi], druz, dzur, drur, row, S_, Hz, Hr);
       if constexpr (kWide<T>) {
         if (link) {
@@ -364,14 +316,6 @@ __device__ __forceinline__ void lbm_tile(const InstDesc* __restrict__ descs,
 #pragma unroll
           for (int i = 0; i < 9; ++i) sFs[i * G::nS + si] = sFs[i * G::nS + si] + h[i];
         }
-      }
-    }
-    if constexpr (MODE == 3) {
-      if (!ax && lr >= 1 && lr <= BR && lc >= 1 && lc <= BZ && k0 + lc - 1 < Nz) {
-        C* o = inter + (size_t)j * P + (k0 + lc - 1);
-        o[I_G1 * iplane] = C(0);
-        o[I_G2 * iplane] = C(0);
-        o[I_G3 * iplane] = C(0);
       }
     }
     sS[si] = S_;
@@ -434,14 +378,6 @@ __device__ __forceinline__ void lbm_tile(const InstDesc* __restrict__ descs,
   });
 }
 
-template <class S, int BZ, int BR, int MODE>
-__global__ void __launch_bounds__(NT, (MinBlocks<S, typename Store<S>::T, BZ, BR>::value)) lbm_kernel(
-    const InstDesc* __restrict__ descs, const int* __restrict__ tile_inst, int toff, int parity,
-    typename Store<S>::C* __restrict__ inter, size_t iplane) {
-  lbm_tile<S, typename Store<S>::T, BZ, BR, MODE>(descs, tile_inst, blockIdx.x + toff, parity, inter,
-                                                  iplane);
-}
-
 // The timestep as a persistent grid (as many CTAs as fit on the GPU at once):
 // CTAs take tiles from a counter in the order of the tile list until none is
 // left, so uneven lattices and ragged tiles leave no partial last wave.
@@ -465,13 +401,13 @@ __global__ void __launch_bounds__(NT, (MinBlocks<S, T, BZ, BR>::value)) lbm_pers
     __syncthreads();
     const int t = s_tile;
     if (t >= ntiles) return;
-    lbm_tile<S, T, BZ, BR, 0>(descs, tile_inst, t, parity, nullptr, 0, step);
+    lbm_tile<S, T, BZ, BR>(descs, tile_inst, t, parity, step);
     __syncthreads();
   }
 }
 
 // ------------------------------------------------------------ split schedule --
-// The same update as lbm_kernel MODE 0 in two kernels, so that the heavy
+// The same update as lbm_persistent in two kernels, so that the heavy
 // per-site chain runs once per site instead of on a halo of 3:
 //   force_kernel  : psi tile + 4, d_r psi on tile + 2, 1D d_r psi on tile
 //                   (z + 2); per site of the tile the moments, forces, u and u^eq,
@@ -493,7 +429,7 @@ struct GeoA {
 
 template <class S, int BZ, int BR>
 __global__ void __launch_bounds__(NT) force_kernel(const InstDesc* __restrict__ descs,
-                                                   const int* __restrict__ tile_inst, int toff,
+                                                   const int* __restrict__ tile_inst,
                                                    int parity) {
   using C = typename Store<S>::C;
   using T = typename Store<S>::T;
@@ -504,7 +440,7 @@ __global__ void __launch_bounds__(NT) force_kernel(const InstDesc* __restrict__ 
   T* sPsi = reinterpret_cast<T*>(smem_raw + G::int_bytes);
   T* sDr = sPsi + G::nP;
   T* sD1 = sDr + G::nD;
-  const Tile Tl = tile_of(descs, tile_inst, blockIdx.x + toff, BZ, BR);
+  const Tile Tl = tile_of(descs, tile_inst, blockIdx.x, BZ, BR);
   const InstDesc& D = descs[Tl.inst];
   const int Nz = D.Nz, Nr = D.Nr, P = D.P, k0 = Tl.k0, j0 = Tl.j0;
   const size_t plane = (size_t)P * Nr;
@@ -574,7 +510,7 @@ struct GeoB {
 
 template <class S, int BZ, int BR>
 __global__ void __launch_bounds__(NT) stream_kernel(const InstDesc* __restrict__ descs,
-                                                    const int* __restrict__ tile_inst, int toff,
+                                                    const int* __restrict__ tile_inst,
                                                     int parity, int* __restrict__ ctr) {
   const uint32_t step = ctr ? (uint32_t)ctr[2 + parity] : 0u;
   if (ctr && blockIdx.x == 0 && threadIdx.x == 0) ctr[2 + (parity ^ 1)] = (int)(step + 1);
@@ -590,7 +526,7 @@ __global__ void __launch_bounds__(NT) stream_kernel(const InstDesc* __restrict__
   T* sHz = sS + G::nS;
   T* sHr = sHz + G::nS;
   T* sFs = sHr + G::nS;
-  const Tile Tl = tile_of(descs, tile_inst, blockIdx.x + toff, BZ, BR);
+  const Tile Tl = tile_of(descs, tile_inst, blockIdx.x, BZ, BR);
   const InstDesc& D = descs[Tl.inst];
   const int Nz = D.Nz, Nr = D.Nr, P = D.P, k0 = Tl.k0, j0 = Tl.j0;
   const size_t plane = (size_t)P * Nr;
@@ -803,41 +739,29 @@ cudaError_t once_per_device(DeviceOnce& st, F&& init, int* grid_cap = nullptr) {
   return st.err[dev];
 }
 
-template <class S, class T, int BZ, int BR, int MODE>
-cudaError_t launch_t(const InstDesc* d, const int* ti, int ntiles, int toff, int parity,
-                     cudaStream_t s, void* inter = nullptr, size_t iplane = 0, int* ctr = nullptr) {
-  using C = typename Store<S>::C;
+template <class S, class T, int BZ, int BR>
+cudaError_t launch_t(const InstDesc* d, const int* ti, int ntiles, int parity, cudaStream_t s, int* ctr) {
   constexpr size_t smem = Geo<T, BZ, BR>::bytes;
   static DeviceOnce st;
   int grid_cap = 0;
   const cudaError_t ie = once_per_device(st, [](int dev, int* cap) {
-    cudaError_t e = cudaFuncSetAttribute(lbm_kernel<S, BZ, BR, MODE>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess && MODE == 0)
-      e = cudaFuncSetAttribute(lbm_persistent<S, T, BZ, BR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem);
-    if (e == cudaSuccess && MODE == 0) {
-      int sms = 0, per_sm = 0;
-      e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lbm_persistent<S, T, BZ, BR>, NT, smem);
-      *cap = sms * (per_sm > 0 ? per_sm : 1);
-    }
+    cudaError_t e = cudaFuncSetAttribute(lbm_persistent<S, T, BZ, BR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    int sms = 0, per_sm = 0;
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lbm_persistent<S, T, BZ, BR>, NT, smem);
+    *cap = sms * (per_sm > 0 ? per_sm : 1);
     return e;
   }, &grid_cap);
   if (ie != cudaSuccess) return ie;
-  if (MODE == 0 && ctr && toff == 0) {
-    const int grid = ntiles < grid_cap ? ntiles : grid_cap;
-    lbm_persistent<S, T, BZ, BR><<<grid, NT, smem, s>>>(d, ti, ntiles, parity, ctr);
-  } else {
-    lbm_kernel<S, BZ, BR, MODE><<<ntiles, NT, smem, s>>>(d, ti, toff, parity, static_cast<C*>(inter), iplane);
-  }
+  lbm_persistent<S, T, BZ, BR><<<ntiles < grid_cap ? ntiles : grid_cap, NT, smem, s>>>(d, ti, ntiles, parity, ctr);
   return cudaGetLastError();
 }
 
 template <class S, int BZ, int BR>
-cudaError_t launch_split_t(const InstDesc* d, const int* ti, int ntiles, int toff, int parity,
-                           cudaStream_t s, int* ctr) {
+cudaError_t launch_split_t(const InstDesc* d, const int* ti, int ntiles, int parity, cudaStream_t s,
+                           int* ctr) {
   using T = typename Store<S>::T;
   constexpr size_t sa = GeoA<T, BZ, BR>::bytes, sbb = GeoB<T, BZ, BR>::bytes;
   static DeviceOnce st;
@@ -850,14 +774,22 @@ cudaError_t launch_split_t(const InstDesc* d, const int* ti, int ntiles, int tof
     return e;
   });
   if (ie != cudaSuccess) return ie;
-  force_kernel<S, BZ, BR><<<ntiles, NT, sa, s>>>(d, ti, toff, parity);
-  stream_kernel<S, BZ, BR><<<ntiles, NT, sbb, s>>>(d, ti, toff, parity, ctr);
+  force_kernel<S, BZ, BR><<<ntiles, NT, sa, s>>>(d, ti, parity);
+  stream_kernel<S, BZ, BR><<<ntiles, NT, sbb, s>>>(d, ti, parity, ctr);
   return cudaGetLastError();
 }
+
+template <class S> struct StorageOf;
+template <> struct StorageOf<float> { static constexpr int value = AMLBM_STORE_F32; };
+template <> struct StorageOf<__half> { static constexpr int value = AMLBM_STORE_F16; };
+template <> struct StorageOf<__nv_bfloat16> { static constexpr int value = AMLBM_STORE_BF16; };
 
 // Tile shapes compiled for each storage form.
 struct TileEntry { int storage, sched, tz, tr; };
 #define AMLBM_TILES_16(ST)                                                                    \
+  {ST, SCHED_FUSED, 26, 4}, {ST, SCHED_FUSED, 26, 5}, {ST, SCHED_FUSED, 26, 6},               \
+  {ST, SCHED_FUSED, 26, 7}, {ST, SCHED_FUSED, 26, 8}, {ST, SCHED_FUSED, 26, 9},               \
+  {ST, SCHED_FUSED, 26, 10},                                                                  \
   {ST, SCHED_FUSED, 26, 16}, {ST, SCHED_FUSED, 32, 16}, {ST, SCHED_FUSED, 64, 8},             \
   {ST, SCHED_FUSED, 58, 8}, {ST, SCHED_FUSED, 32, 8}, {ST, SCHED_FUSED, 32, 32},              \
   {ST, SCHED_FUSED, 64, 16}, {ST, SCHED_SPLIT, 32, 16}, {ST, SCHED_SPLIT, 64, 8},             \
@@ -870,18 +802,16 @@ constexpr TileEntry kTiles[] = {
 #undef AMLBM_TILES_16
 
 template <class S>
-cudaError_t dispatch(bool macro, int sched, int tz, int tr, const InstDesc* d, const int* ti, int nt,
-                     int toff, int par, cudaStream_t s, int* ctr) {
+cudaError_t dispatch(int sched, int tz, int tr, const InstDesc* d, const int* ti, int nt,
+                     int par, cudaStream_t s, int* ctr) {
   using T = typename Store<S>::T;
   if (nt <= 0) return cudaSuccess;
-  if constexpr (!std::is_same<S, double>::value) {  // the FP64 form has its own (launch_step, launch_macro)
-    if (macro) {
-      if (tz == 26 && tr == 16) return launch_t<S, T, 26, 16, 1>(d, ti, nt, toff, par, s);
-      return cudaErrorInvalidValue;
-    }
+  if constexpr (!std::is_same<S, double>::value) {  // the FP64 form has its own (launch_step)
+    if (sched == SCHED_FUSED && tz == kRowWidth && row_rows_ok(tr))
+      return launch_step_row(StorageOf<S>::value, tr, d, ti, nt, par, s, ctr);
     if (sched == SCHED_SPLIT) {
 #define AMLBM_SPLIT(TZ, TR) \
-  if (tz == TZ && tr == TR) return launch_split_t<S, TZ, TR>(d, ti, nt, toff, par, s, ctr);
+  if (tz == TZ && tr == TR) return launch_split_t<S, TZ, TR>(d, ti, nt, par, s, ctr);
       AMLBM_SPLIT(32, 8)
       AMLBM_SPLIT(64, 8)
       AMLBM_SPLIT(32, 16)
@@ -891,7 +821,7 @@ cudaError_t dispatch(bool macro, int sched, int tz, int tr, const InstDesc* d, c
     }
   }
 #define AMLBM_TILE(TZ, TR) \
-  if (tz == TZ && tr == TR) return launch_t<S, T, TZ, TR, 0>(d, ti, nt, toff, par, s, nullptr, 0, ctr);
+  if (tz == TZ && tr == TR) return launch_t<S, T, TZ, TR>(d, ti, nt, par, s, ctr);
   AMLBM_TILE(32, 8)
   AMLBM_TILE(64, 8)
   AMLBM_TILE(58, 8)
@@ -907,14 +837,14 @@ cudaError_t dispatch(bool macro, int sched, int tz, int tr, const InstDesc* d, c
   return cudaErrorInvalidValue;
 }
 
-cudaError_t dispatch_storage(int storage, bool macro, int sched, int tz, int tr, const InstDesc* d,
-                             const int* ti, int nt, int toff, int par, cudaStream_t s, int* ctr) {
+cudaError_t dispatch_storage(int storage, int sched, int tz, int tr, const InstDesc* d,
+                             const int* ti, int nt, int par, cudaStream_t s, int* ctr) {
   switch (storage) {
-    case AMLBM_STORE_F64: return dispatch<double>(macro, sched, tz, tr, d, ti, nt, toff, par, s, ctr);
-    case AMLBM_STORE_F32: return dispatch<float>(macro, sched, tz, tr, d, ti, nt, toff, par, s, ctr);
-    case AMLBM_STORE_F16: return dispatch<__half>(macro, sched, tz, tr, d, ti, nt, toff, par, s, ctr);
+    case AMLBM_STORE_F64: return dispatch<double>(sched, tz, tr, d, ti, nt, par, s, ctr);
+    case AMLBM_STORE_F32: return dispatch<float>(sched, tz, tr, d, ti, nt, par, s, ctr);
+    case AMLBM_STORE_F16: return dispatch<__half>(sched, tz, tr, d, ti, nt, par, s, ctr);
     case AMLBM_STORE_BF16:
-      return dispatch<__nv_bfloat16>(macro, sched, tz, tr, d, ti, nt, toff, par, s, ctr);
+      return dispatch<__nv_bfloat16>(sched, tz, tr, d, ti, nt, par, s, ctr);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -942,40 +872,29 @@ int tile_list(int storage, int sched, int* tz, int* tr, int cap) {
 }
 
 cudaError_t launch_step(int storage, int sched, int form, bool odd, int tz, int tr, const InstDesc* d, const int* ti,
-                        int nt, int toff, int parity, cudaStream_t s, int* ctr) {
-  if (sched == SCHED_PAIR) {
-    if (toff != 0) return cudaErrorInvalidValue;
-    return launch_step_pair(storage, form, odd, tz, tr, d, ti, nt, parity, s, ctr);
-  }
-  if (sched == SCHED_SPLIT && storage == AMLBM_STORE_F64) {
-    if (toff != 0) return cudaErrorInvalidValue;
+                        int nt, int parity, cudaStream_t s, int* ctr) {
+  if (!ctr) return cudaErrorInvalidValue;
+  if (sched == SCHED_PAIR) return launch_step_pair(storage, form, odd, tz, tr, d, ti, nt, parity, s, ctr);
+  if (sched == SCHED_SPLIT && storage == AMLBM_STORE_F64)
     return launch_step_split64(tz, tr, d, ti, nt, parity, s, ctr);
-  }
-  return dispatch_storage(storage, false, sched, tz, tr, d, ti, nt, toff, parity, s, ctr);
+  return dispatch_storage(storage, sched, tz, tr, d, ti, nt, parity, s, ctr);
 }
 cudaError_t launch_macro(int storage, int tz, int tr, const InstDesc* d, const int* ti, int nt,
                          int toff, int parity, cudaStream_t s) {
   if (storage == AMLBM_STORE_F64) return launch_readback64(tz, tr, d, ti, nt, toff, parity, s);
-  return dispatch_storage(storage, true, SCHED_FUSED, tz, tr, d, ti, nt, toff, parity, s, nullptr);
+  return launch_readback_row(storage, d, ti, nt, toff, parity, s);
 }
 
 cudaError_t macro_preload(int storage, int rz, int rr) {
-  cudaFuncAttributes a;
-  switch (storage) {  // the read-back tiles of rb_tile()
-    case AMLBM_STORE_F64: return readback64_preload(rz, rr);
-    case AMLBM_STORE_F32: return cudaFuncGetAttributes(&a, lbm_kernel<float, 26, 16, 1>);
-    case AMLBM_STORE_F16: return cudaFuncGetAttributes(&a, lbm_kernel<__half, 26, 16, 1>);
-    case AMLBM_STORE_BF16: return cudaFuncGetAttributes(&a, lbm_kernel<__nv_bfloat16, 26, 16, 1>);
-    default: return cudaErrorInvalidValue;
-  }
+  return storage == AMLBM_STORE_F64 ? readback64_preload(rz, rr) : readback_row_preload(storage);
 }
 
 cudaError_t launch_step_inter(int storage, int tz, int tr, const InstDesc* d, const int* ti, int nt, void* inter,
                               size_t plane, void* fstar, cudaStream_t s) {
   if (storage == AMLBM_STORE_F64)
     return launch_step_inter64(tz, tr, d, ti, nt, static_cast<double*>(inter), plane, static_cast<double*>(fstar), s);
-  if (storage == AMLBM_STORE_F32 && tz == 32 && tr == 8)
-    return launch_t<float, F1, 32, 8, 3>(d, ti, nt, 0, 0, s, inter, plane);
+  if (storage == AMLBM_STORE_F32 && tz == kRowWidth)
+    return launch_step_inter_row(tr, d, ti, nt, static_cast<float*>(inter), plane, s);
   return cudaErrorInvalidValue;
 }
 

@@ -41,9 +41,8 @@ def run(specs, storage, steps, **how):
 def test_strips_equal_fused_bitwise(Nz, Nr, storage, kw):
     spec = [amlbm.InstanceSpec(Nz, Nr, 0.9, -4.9, **kw)]
     ref, _ = run(spec, storage, 20, tile=(32, 8), schedule="fused")
-    for rows in (None, 2, 6, 18, 66):
-        got, kind = run(spec, storage, 20, **(dict(tile=(48, rows), schedule="pair") if rows else {}))
-        assert kind[0] == "pair" and kind[1][0] == 48
+    for rows in (2, 6, 18, 66):
+        got, kind = run(spec, storage, 20, tile=(48, rows), schedule="pair")
         for a, b in zip(ref, got):
             assert np.array_equal(a, b), (kind, np.abs(a - b).max())
 
@@ -53,9 +52,10 @@ def test_strips_equal_fused_bitwise(Nz, Nr, storage, kw):
 @pytest.mark.parametrize("Nz,Nr", [(1, 8), (3, 5), (47, 9), (49, 4), (63, 33), (65, 20), (97, 61), (255, 65)])
 def test_odd_widths_equal_fused_bitwise(Nz, Nr, kw):
     """FP32 lattices of odd width, alone and beside even ones (among them one that is a
-    single strip): the library's own choice; a requested pair schedule refuses them."""
-    odd = amlbm.InstanceSpec(Nz, Nr, 0.9, -4.9, **kw)
-    for specs in ([odd], [amlbm.InstanceSpec(64, 12, 0.9, -4.9), odd, amlbm.InstanceSpec(150, 31, 1.0, -5.0)]):
+    single strip): the library's own choice for batches of some size (the last lattice); a
+    requested pair schedule refuses them."""
+    odd, large = amlbm.InstanceSpec(Nz, Nr, 0.9, -4.9, **kw), amlbm.InstanceSpec(512, 160, 0.9, -4.9, **kw)
+    for specs in ([odd, large], [amlbm.InstanceSpec(64, 12, 0.9, -4.9), odd, amlbm.InstanceSpec(150, 31, 1.0, -5.0), large]):
         ref, _ = run(specs, "f32", 20, tile=(32, 8), schedule="fused")
         got, kind = run(specs, "f32", 20)
         assert kind[0] == "pair" and kind[1][0] == 48
@@ -71,7 +71,7 @@ def test_strips_of_mixed_lattices_equal_fused_bitwise(storage):
     the options), and a uniform batch large enough for several rounds of strips."""
     mixed = [amlbm.InstanceSpec(40, 20, 0.9, -5.0), amlbm.InstanceSpec(130, 33, 1.0, -4.8, wall="noslip"),
              amlbm.InstanceSpec(66, 47, 0.8, -5.0, forcing="guo"), amlbm.InstanceSpec(64, 9, 1.1, -4.9, axisym=False),
-             amlbm.InstanceSpec(100, 50, 0.9, -5.0, shift="equilibrium")]
+             amlbm.InstanceSpec(100, 50, 0.9, -5.0, shift="equilibrium"), amlbm.InstanceSpec(512, 160, 0.9, -5.0)]
     many = [amlbm.InstanceSpec(2 * (30 + 7 * k % 90), 20 + 11 * k % 101, 0.9, -4.9) for k in range(120)]
     for specs in (mixed, many):
         ref, _ = run(specs, storage, 10, tile=(26, 16), schedule="fused")
