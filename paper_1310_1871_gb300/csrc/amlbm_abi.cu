@@ -316,11 +316,11 @@ Layout make_layout(const std::vector<amlbm_instance>& inst, int storage, int tz,
     L.rb_ntiles += amlbm::tiles_along_z(sched, rz, I.Nz) * ((I.Nr + rr - 1) / rr);
     L.maxN = std::max(L.maxN, I.Nz * I.Nr);
     L.maxNz = std::max(L.maxNz, I.Nz);
-    L.diag_nblk = std::max(L.diag_nblk, amlbm::diag_blocks(I.Nz, I.Nr));
-    L.all_nblk += amlbm::diag_blocks(I.Nz, I.Nr);
+    L.diag_nblk = std::max(L.diag_nblk, amlbm::diag_blocks(I.Nz, I.Nr, (long long)I.Nz * I.Nr));
     L.sumN += (long long)I.Nz * I.Nr;
     L.sumNz += I.Nz;
   }
+  for (const auto& I : inst) L.all_nblk += amlbm::diag_blocks(I.Nz, I.Nr, L.sumN);
   L.desc = take(n * sizeof(InstDesc));
   L.tiles = take((size_t)L.ntiles * sizeof(int));
   L.rb_tiles = take((size_t)L.rb_ntiles * sizeof(int));
@@ -576,7 +576,7 @@ int batch_build(const std::vector<amlbm_instance>& inst, const amlbm_tune* tune,
   std::vector<int> blkjob;
   blkjob.reserve(L.all_nblk);
   for (int i = 0; i < b->n; ++i)
-    for (int q = 0; q < amlbm::diag_blocks(inst[i].Nz, inst[i].Nr); ++q) blkjob.push_back(i);
+    for (int q = 0; q < amlbm::diag_blocks(inst[i].Nz, inst[i].Nr, L.sumN); ++q) blkjob.push_back(i);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(b->arena + L.diag_blkjob, blkjob.data(), blkjob.size() * sizeof(int),
                         cudaMemcpyHostToDevice, b->stream);
@@ -779,7 +779,7 @@ int diag_all_host(amlbm_batch* b, const amlbm_diag_params* dp, amlbm_diag* out) 
     amlbm::diag_job_constants(J);
     J.inst = k;
     J.blk0 = blk;
-    J.nblk = amlbm::diag_blocks(d.Nz, d.Nr);
+    J.nblk = amlbm::diag_blocks(d.Nz, d.Nr, b->sites);
     J.col0 = col;
     blk += J.nblk;
     col += d.Nz;
@@ -841,7 +841,7 @@ int diag_host(amlbm_batch* b, int k, const amlbm_diag_params* dp, amlbm_diag* ou
   double* part = reinterpret_cast<double*>(b->arena + b->L.diag_part);
   double* cols = reinterpret_cast<double*>(b->arena + b->L.diag_cols);
   double* res = reinterpret_cast<double*>(b->arena + b->L.diag_out);
-  const int nblk = amlbm::diag_blocks(d.Nz, d.Nr);
+  const int nblk = amlbm::diag_blocks(d.Nz, d.Nr, (long long)d.Nz * d.Nr);
   const cudaError_t e = amlbm::launch_diag(b->storage, b->d_desc, k, d.Nz, d.Nr, b->parity, p.zc, p.R,
                                            p.rho_l, p.rho_v, part, nblk, cols, res, b->stream);
   if (e != cudaSuccess) return fail(AMLBM_ECUDA, std::string("diag kernels: ") + cudaGetErrorString(e));

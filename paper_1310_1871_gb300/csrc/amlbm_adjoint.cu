@@ -551,7 +551,7 @@ AdjLayout adj_layout(const amlbm::CtxInfo& ci, const amlbm_adjoint_problem& p) {
   L.arr = take((size_t)kAdjArrays * plane * cb);
   L.acc = take(2 * plane * sizeof(double));
   L.rho0 = take((size_t)ci.Nz * ci.Nr * sizeof(double));
-  const int nblk = amlbm::diag_blocks(ci.Nz, ci.Nr);
+  const int nblk = amlbm::diag_blocks(ci.Nz, ci.Nr, (long long)ci.Nz * ci.Nr);
   L.red = take((size_t)(std::max(L.nred * 34, 8 * nblk + ci.Nz + 16) + 64) * sizeof(double));
   L.descs = take((size_t)L.nbuf * L.nseg * sizeof(InstDesc));
   L.tiles = take((size_t)L.ntiles * sizeof(int));
@@ -653,7 +653,7 @@ int run(amlbm_ctx* ctx, const amlbm_adjoint_problem* p, void* ws, size_t ws_byte
     {
       double a2 = 0.0;
       if (p->objective == AMLBM_OBJ_A2SQ) {
-        const int nblk = diag_blocks(Nz, Nr);
+        const int nblk = diag_blocks(Nz, Nr, (long long)Nz * Nr);
         ADJ_CK(launch_diag(ci.storage, ci.d_desc, 0, Nz, Nr, ci.parity ^ (p->T & 1), p->zc, p->obj_R,
                            p->rho_l, p->rho_v, redbuf, nblk, redbuf + 8 * nblk, redbuf + 8 * nblk + Nz, s));
         ADJ_CK(cudaMemcpyAsync(&a2, redbuf + 8 * nblk + Nz + 5, sizeof(double), cudaMemcpyDeviceToHost, s));

@@ -141,11 +141,12 @@ inline void inter_tile(int storage, int Nz, int Nr, int* tz, int* tr) {
 }
 // Diagnostics (amlbm_diag.cu) of the state whose rho / u the read-back kernel
 // has written: partial sums into `partials` (nblk x 8 doubles) and the Nz column
-// radii into `cols`, then a single-block pass into out[16].
+// radii into `cols`, then one block's pass into out[16].
 cudaError_t launch_diag(int storage, const InstDesc* d_desc, int inst, int Nz, int Nr,
                         int parity, double zc, double R, double rho_l, double rho_v,
                         double* partials, int nblk, double* cols, double* out, cudaStream_t s);
-int diag_blocks(int Nz, int Nr);
+// Blocks of one lattice in a pass over `sites` sites (its own, or the whole batch's).
+int diag_blocks(int Nz, int Nr, long long sites);
 // Loads the code of the single-lattice diagnostics kernels on the current device
 // (the CUDA runtime otherwise loads it at their first launch).
 cudaError_t diag_preload();

@@ -103,7 +103,7 @@ extern "C" int amlbm_diagnostics_noalloc(amlbm_ctx* ctx, const amlbm_diag_params
     return set_error(AMLBM_EINVAL, "amlbm_diagnostics_noalloc: Nz = " + std::to_string(Nz) +
                                         " exceeds the static scratch limit AMLBM_NOALLOC_MAX_NZ = " +
                                         std::to_string(AMLBM_NOALLOC_MAX_NZ));
-  const int nblk = amlbm::diag_blocks(Nz, Nr);
+  const int nblk = amlbm::diag_blocks(Nz, Nr, (long long)Nz * Nr);
   if (nblk > kMaxBlocks)
     return set_error(AMLBM_EINVAL, "amlbm_diagnostics_noalloc: lattice too large");
   double* scratch = nullptr;
