@@ -176,8 +176,8 @@ int pick_strip(const std::vector<amlbm_instance>& inst) {
 //
 // FP64: the two kernels of amlbm_step_split64.cu, on the largest tile that still keeps
 // the 152 SMs busy.  Measured (us per step on 8 x 4 / 16 x 8 / 32 x 8 / 32 x 16 tiles):
-// 64 x 32 11.2 / 16.5 / 22.4 / 37.3 (the recomputing kernels before: 38); 192 x 96 17.8 /
-// 16.1 / 22.5 / 37.7; 256 x 128 26.1 / 24.2 / 23.0 / 38.3; 512 x 256 90 / 68 / 68.0 / 66.5;
+// 64 x 32 9.2 / 14.4 / 21.1 / 36.0 (the recomputing kernels before: 38); 192 x 96 16.6 /
+// 14.7 / 21.2 / 35.8; 256 x 128 26.1 / 24.2 / 21.0 / 38.3; 512 x 256 90 / 68 / 68.0 / 66.5;
 // 1024 x 512 338 / 250 / 227 / 218 (before: 394); 330,400 sites in 25 lattices 217 / 168 /
 // 158.5 / 164.5.
 //

@@ -21,8 +21,15 @@
 // that of every other FP64 schedule, operation for operation, so the states are
 // bit-identical.  It takes every lattice the fused schedule takes.
 //
-// Measured (GB300, one step): see the figures beside pick_tile (amlbm_abi.cu), which
-// chooses the tile.
+// On small grids each kernel lets the next start as soon as it has begun to read
+// (pdl_trigger): its blocks then wait beside this one's with their index and row
+// constants ready.  us per step without / with it: 64 x 32 (64 blocks of 8 x 4) 10.7 / 9.2,
+// 128 x 64 (256) 12.7 / 11.0, 192 x 80 (480) 17.6 / 16.2, 256 x 128 (128 of 32 x 8) 22.7 / 21.0,
+// 384 x 200 (300) 37.1 / 35.8.  Beyond, the next kernel's blocks crowd onto the SMs that are
+// free first: 192 x 120 (180 of 16 x 8) 23.6 / 27.3, 512 x 200 (400 of 32 x 8) 52.2 / 65.7.  The
+// adjoint's forward steps (MODE 3) never do: they run beside another stream, whose kernels
+// need the room (gradient of 256 x 128 over 50 steps 3.77 ms, with it 4.15).
+// The figures for every tile stand beside pick_tile (amlbm_abi.cu), which chooses it.
 
 #include <stdint.h>
 
@@ -49,6 +56,8 @@ struct Geo64 {
   static constexpr int ROLES = SITES >= 256 ? 1 : SITES >= 128 ? 2 : 4;
   static constexpr int NT = SITES * ROLES < 256 ? SITES * ROLES : 256;
   static_assert(SITES % 32 == 0 && (ROLES == 1 || NT == SITES * ROLES), "a role is whole warps");
+  // the largest grid that starts the next kernel early
+  static constexpr unsigned kEarly = ROLES == 4 ? 512 : SITES == 256 ? 304 : 152;
   static constexpr int PZ = BZ + 8, PR = BR + 8;  // psi
   static constexpr int DZ = BZ + 4, DR = BR + 4;  // isotropic d_r psi
   static constexpr int FZ = BZ + 6, FR = BR + 6;  // u
@@ -68,6 +77,13 @@ __device__ __forceinline__ void for_sites(F&& body) {
 __host__ __device__ constexpr int role_of(int i, int roles) {
   return (i == 0 || i == 1 || i == 3 ? 0 : i == 2 || i == 4 ? 1 : i == 5 || i == 7 ? 2 : 3) % roles;
 }
+
+// In f64_stream the directions are split by the terms of moment0, of which each role adds
+// its own (64 x 32: 0.2 us per step): part p, of role p % roles.
+__host__ __device__ constexpr int part_of(int i) {
+  return i == 0 || i == 2 || i == 4 ? 0 : i == 1 || i == 3 ? 1 : i == 5 || i == 6 ? 2 : 3;
+}
+__host__ __device__ constexpr int pull_role(int i, int roles) { return part_of(i) % roles; }
 
 // body(integral_constant role) for this thread's role (uniform in a warp)
 template <int ROLES, class F>
@@ -118,6 +134,7 @@ __global__ void __launch_bounds__(Geo64<BZ, BR>::NT) f64_force(const InstDesc* _
   if (threadIdx.x < BR) sRow[threadIdx.x] = row_of(q, j0 + (int)threadIdx.x, D.k64[K_R0]);
   __syncthreads();
   pdl_wait();  // everything above reads only what creation wrote
+  if (MODE != 3 && gridDim.x <= G::kEarly) pdl_trigger();
 
   for_sites<G::NT, G::PR, G::PZ>([&](int lr, int lc) { sPsi[lr * G::PZ + lc] = T{psin[sOff[lr] + sCol[lc]]}; });
   __syncthreads();
@@ -261,7 +278,7 @@ __global__ void __launch_bounds__(Geo64<BZ, BR>::NT) f64_stream(const InstDesc* 
   __shared__ T sUz[G::FR * G::FZ], sUr[G::FR * G::FZ];
   __shared__ T sS[G::SR * G::SZ], sHz[G::SR * G::SZ], sHr[G::SR * G::SZ];
   __shared__ T sB[2][9][G::SZ];  // populations of an inlet row and an outlet row
-  __shared__ T sF[ROLES > 1 ? 9 * G::SITES : 1];  // the arrivals, for rho
+  __shared__ T sF[ROLES > 1 ? 4 * G::SITES : 1];  // the parts of rho
   __shared__ Row<T> sRow[G::SR];
   __shared__ int sCol[G::FZ];
   const int tile = blockIdx.x;
@@ -280,6 +297,7 @@ __global__ void __launch_bounds__(Geo64<BZ, BR>::NT) f64_stream(const InstDesc* 
   if (threadIdx.x < G::SR) sRow[threadIdx.x] = row_of(q, j0 - 1 + (int)threadIdx.x, D.k64[K_R0]);
   __syncthreads();
   pdl_wait();
+  if (MODE != 3 && gridDim.x <= G::kEarly) pdl_trigger();
   if (ctr && blockIdx.x == 0 && threadIdx.x == 0) ctr[2 + (parity ^ 1)] = ctr[2 + parity] + 1;
 
   // u on the tile + 3.  Ghost columns at the z walls: u odd.  Ghost rows (depth 2):
@@ -395,7 +413,7 @@ __global__ void __launch_bounds__(Geo64<BZ, BR>::NT) f64_stream(const InstDesc* 
       with_role<ROLES>(role, [&](auto R) {
 #pragma unroll
         for (int i = 0; i < 9; ++i)
-          if (role_of(i, ROLES) == R.value)
+          if (pull_role(i, ROLES) == R.value)
             fn[i] = T{fs[i * plane + (j - cr_(i)) * P + (cz_(i) == 0 ? k : cz_(i) > 0 ? km : kp)]};
       });
     }
@@ -407,7 +425,7 @@ __global__ void __launch_bounds__(Geo64<BZ, BR>::NT) f64_stream(const InstDesc* 
           if (ax) {
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
-              if (role_of(i, ROLES) != R.value) continue;
+              if (pull_role(i, ROLES) != R.value) continue;
               const int si = (lr + 1 - cr_(i)) * G::SZ + (lc + 1 - cz_(i));
               fn[i] = add_source(i, fn[i], sS[si], sHz[si], sHr[si]);
             }
@@ -415,7 +433,7 @@ __global__ void __launch_bounds__(Geo64<BZ, BR>::NT) f64_stream(const InstDesc* 
         } else {
 #pragma unroll
           for (int i = 0; i < 9; ++i) {
-            if (role_of(i, ROLES) != R.value) continue;
+            if (pull_role(i, ROLES) != R.value) continue;
             // where the population arriving in direction i leaves from: row sj, column sk,
             // direction ii, which is i with the flagged components reversed
             int sj = j - cr_(i), sk = cz_(i) == 0 ? k : cz_(i) > 0 ? km : kp, ii = i;
@@ -449,24 +467,28 @@ __global__ void __launch_bounds__(Geo64<BZ, BR>::NT) f64_stream(const InstDesc* 
           const int di = (lr + 1) * G::SZ + (lc + 1);
 #pragma unroll
           for (int i = 0; i < 9; ++i)
-            if (role_of(i, ROLES) == R.value) fn[i] = add_source(i, fn[i], sS[di], sHz[di], sHr[di]);
+            if (pull_role(i, ROLES) == R.value) fn[i] = add_source(i, fn[i], sS[di], sHz[di], sHr[di]);
         }
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
-          if (role_of(i, ROLES) != R.value) continue;
+          if (pull_role(i, ROLES) != R.value) continue;
           fout[i * plane + o] = fn[i].v;
-          if constexpr (ROLES > 1) sF[i * G::SITES + t] = fn[i];
+        }
+        if constexpr (ROLES > 1) {
+          if (R.value == 0) sF[t] = fn[0] + (fn[2] + fn[4]);
+          if (R.value == 1 % ROLES) sF[G::SITES + t] = fn[1] + fn[3];
+          if (R.value == 2 % ROLES) sF[2 * G::SITES + t] = fn[5] + fn[6];
+          if (R.value == 3 % ROLES) sF[3 * G::SITES + t] = fn[7] + fn[8];
         }
       });
     }
-    if constexpr (ROLES > 1) {
-      __syncthreads();
-      if (role == 0) {
-#pragma unroll
-        for (int i = 0; i < 9; ++i) fn[i] = sF[i * G::SITES + t];
-      }
+    if constexpr (ROLES > 1) __syncthreads();
+    if (in && role == 0) {
+      T rho;
+      if constexpr (ROLES > 1) rho = sF[t] + (sF[G::SITES + t] + (sF[2 * G::SITES + t] + sF[3 * G::SITES + t]));
+      else rho = moment0(fn);
+      psout[o] = psi_of(q, rho).v;
     }
-    if (in && role == 0) psout[o] = psi_of(q, moment0(fn)).v;
   }
 }
 
