@@ -125,7 +125,7 @@ long long count_tiles(const std::vector<amlbm_instance>& inst, int tz, int tr) {
 // rows of psi, 0.65 for the next 4, then n + 2 whole rows, four at a time.  Measured on
 // the 64-drop sweep of 835,240 sites (us per step): H = 18 21.5 (1157 strips, one round),
 // 10 28.7, 20 24.2, 26 27.1.
-int pick_strip(const std::vector<amlbm_instance>& inst) {
+int pick_strip(const std::vector<amlbm_instance>& inst, double* units, long long* count) {
   constexpr int kPlaces = 8 * 152;
   auto cost = [](int rows) { return 4.6 + 4.0 * ((rows + 2 + 3) / 4); };
   int best = 2, max_rows = 0;
@@ -166,11 +166,15 @@ int pick_strip(const std::vector<amlbm_instance>& inst) {
     if (t < least) {
       least = t;
       best = h;
+      *count = strips;
     }
     if (h >= max_rows) break;
   }
+  *units = least;
   return best;
 }
+
+int resolve_shift(const amlbm_bc& bc);
 
 // Schedule and tile when the caller gives none.
 //
@@ -182,8 +186,11 @@ int pick_strip(const std::vector<amlbm_instance>& inst) {
 // 158.5 / 164.5.
 //
 // FP32 arithmetic: the row kernel's tiles while they all run at once (row_height), then
-// the pair schedule's strips where every lattice allows them (pick_strip), else the fused
-// schedule: two rounds of the row kernel's largest tiles (512 x 256: 10.5 us per step; the
+// the pair schedule's strips where every lattice allows them (pick_strip; with the
+// equilibrium shift in 16 bits, whose codec makes a strip's rows longer, 64 x 24 tiles where
+// one or two rounds of them are faster: us per step on strips / tiles, FP16, 512 x 256 14.3 /
+// 14.4, 768 x 256 16.0 / 14.5, three threads of 344,448 sites 22.2 / 20.6, 700 x 700 22.7 / 26.8),
+// else the fused schedule: two rounds of the row kernel's largest tiles (512 x 256: 10.5 us per step; the
 // persistent grid on 26 x 16 14.4), beyond that the persistent grid (1024 x 512: 28.7; rows 36).
 void pick_tile(int storage, const std::vector<amlbm_instance>& inst, int* sched, int* tz, int* tr) {
   if (storage == AMLBM_STORE_F64) {
@@ -202,7 +209,17 @@ void pick_tile(int storage, const std::vector<amlbm_instance>& inst, int* sched,
   if (all_pair_ok(inst, storage == AMLBM_STORE_F32)) {
     *sched = amlbm::SCHED_PAIR;
     *tz = amlbm::kStripWidth;
-    *tr = pick_strip(inst);
+    double units = 0.0;
+    long long strips = 0;
+    *tr = pick_strip(inst, &units, &strips);
+    bool shifted = false;
+    for (const auto& I : inst) shifted = shifted || resolve_shift(I.bc) == 3;
+    const long long rounds = (count_tiles(inst, 64, 24) + 151) / 152;
+    if (shifted && elem_bytes(storage) == 2 && rounds <= 2 &&
+        8.2 + 6.2 * rounds < 0.95 * (1.7 + 1.05 * units) * (strips > 4 * 152 ? 1.16 : 1.0)) {
+      *tz = 64;
+      *tr = 24;
+    }
     return;
   }
   if (count_tiles(inst, amlbm::kRowWidth, amlbm::kRowMaxRows) <= 4 * 152) {

@@ -57,6 +57,14 @@ def test_narrow_periodic_lattices(Nz, Nr):
     same(run(spec, "f32", tile=(32, 8), schedule="fused")[0], run(spec, "f32")[0])
 
 
+def test_choice_in_16_bits_with_the_equilibrium_shift():
+    for Nz, Nr, tile in ((768, 256, (64, 24)), (512, 160, (48, 2)), (700, 700, (48, 10))):
+        spec = amlbm.InstanceSpec(Nz, Nr, 0.9, -4.9, shift="equilibrium")
+        got, kind = run(spec, "f16", 4)
+        assert kind == ("pair", tile)
+        same(run(spec, "f16", 4, tile=(32, 8), schedule="fused")[0], got)
+
+
 @pytest.mark.parametrize("Nz,Nr,kw,tile", [
     (64, 32, {}, ("fused", (26, 4))), (256, 128, {}, ("fused", (26, 9))), (520, 150, {}, ("fused", (26, 10))),
     (520, 152, {}, ("pair", None)), (780, 200, dict(src="link"), ("fused", (26, 10))),
