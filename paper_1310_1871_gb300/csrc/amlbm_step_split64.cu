@@ -16,7 +16,7 @@
 //                Sec. II.E) with the sources of their departure sites, and psi of the
 //                new state
 //
-// 208 FP64 operations per site (exp counts 20) on 32 x 8 tiles, against 472 for the
+// 214 FP64 operations per site (exp counts 20) on 32 x 8 tiles, against 472 for the
 // kernels that recomputed the collision on the streaming halo.  The arithmetic is
 // that of every other FP64 schedule, operation for operation, so the states are
 // bit-identical.  It takes every lattice the fused schedule takes.
@@ -73,10 +73,12 @@ __device__ __forceinline__ void for_sites(F&& body) {
 }
 
 // The role that handles direction i: pairs of opposite directions stay together (they
-// share their parts), the rest population with the first pair.
-__host__ __device__ constexpr int role_of(int i, int roles) {
-  return (i == 0 || i == 1 || i == 3 ? 0 : i == 2 || i == 4 ? 1 : i == 5 || i == 7 ? 2 : 3) % roles;
+// share their parts).  The rest population, which takes what the pairs leave of rho, comes
+// last, from the role of the first pair.
+__host__ __device__ constexpr int pair_of(int i) {
+  return i == 0 || i == 1 || i == 3 ? 0 : i == 2 || i == 4 ? 1 : i == 5 || i == 7 ? 2 : 3;
 }
+__host__ __device__ constexpr int role_of(int i, int roles) { return pair_of(i) % roles; }
 
 // In f64_stream the directions are split by the terms of moment0, of which each role adds
 // its own (64 x 32: 0.2 us per step): part p, of role p % roles.
@@ -112,7 +114,7 @@ __global__ void __launch_bounds__(Geo64<BZ, BR>::NT) f64_force(const InstDesc* _
   using G = Geo64<BZ, BR>;
   constexpr int ROLES = G::ROLES;
   __shared__ T sPsi[G::PR * G::PZ], sDr[G::DR * G::DZ], sD1[BR * G::DZ];
-  __shared__ T sX[ROLES > 1 ? 10 * G::SITES : 1];  // what the roles of a site share
+  __shared__ T sX[ROLES > 1 ? 14 * G::SITES : 1];  // what the roles of a site share
   __shared__ Row<T> sRow[BR];
   __shared__ int sCol[G::PZ], sOff[G::PR];
   const int tile = blockIdx.x + toff;
@@ -156,6 +158,7 @@ __global__ void __launch_bounds__(Geo64<BZ, BR>::NT) f64_force(const InstDesc* _
     const T* dr = sDr + (lr + 2) * G::DZ + (lc + 2);
     const T psi = p[0];
     const Row<T>& row = sRow[lr];
+    double* out = (MODE == 3 ? fstar : f) + o;
     T fv[9], sz, sr, dr0 = lit<T>(0.0), Drr = lit<T>(0.0), Dzr = lit<T>(0.0), rho, jz, jr, inv_rho, Fz, Fr;
     if constexpr (ROLES == 1) {
       if (!in) continue;
@@ -203,7 +206,6 @@ __global__ void __launch_bounds__(Geo64<BZ, BR>::NT) f64_force(const InstDesc* _
         x[9 * NS] = moment_r(fv);
       }
       __syncthreads();
-      if (!in) return;  // one site per thread: nothing follows
       rho = x[6 * NS];
       inv_rho = x[7 * NS];
       jz = x[8 * NS];
@@ -216,51 +218,66 @@ __global__ void __launch_bounds__(Geo64<BZ, BR>::NT) f64_force(const InstDesc* _
       }
       Fz = fma(rho, q.gz, Fz);
     }
-    const T uz = fma(Fz, lit<T>(0.5), jz) * inv_rho, ur = fma(Fr, lit<T>(0.5), jr) * inv_rho;
-    if constexpr (MODE == 1) {
-      const size_t w = (size_t)j * Nz + k;
-      if (role == 0) {
-        static_cast<double*>(D.rho_out)[w] = rho.v;
-        static_cast<double*>(D.uz_out)[w] = uz.v;
-        static_cast<double*>(D.ur_out)[w] = ur.v;
-      }
-    } else {
-      if (role == ROLES - 1) {
-        double* uv = static_cast<double*>(D.uv) + o;
-        uv[0] = uz.v;
-        uv[plane] = ur.v;
-        uv[2 * plane] = rho.v;
-      }
-      if constexpr (MODE == 3) {
-        double* w = inter + o;
+    if (in) {
+      const T uz = fma(Fz, lit<T>(0.5), jz) * inv_rho, ur = fma(Fr, lit<T>(0.5), jr) * inv_rho;
+      if constexpr (MODE == 1) {
+        const size_t w = (size_t)j * Nz + k;
         if (role == 0) {
-          w[I_SZ * iplane] = unscale(sz, 36.0).v;
-          w[I_SR * iplane] = unscale(sr, 36.0).v;
-          w[I_PSI * iplane] = psi.v;
+          static_cast<double*>(D.rho_out)[w] = rho.v;
+          static_cast<double*>(D.uz_out)[w] = uz.v;
+          static_cast<double*>(D.ur_out)[w] = ur.v;
         }
-        if (role == 1 % ROLES) {
-          w[I_DR * iplane] = unscale(dr0, 36.0).v;
-          w[I_DRR * iplane] = unscale(Drr, 1296.0).v;
-          w[I_DZR * iplane] = unscale(Dzr, 144.0).v;
+      } else {
+        if (role == ROLES - 1) {
+          double* uv = static_cast<double*>(D.uv) + o;
+          uv[0] = uz.v;
+          uv[plane] = ur.v;
+          uv[2 * plane] = rho.v;
         }
-        if (role == 2 % ROLES) {
-          w[I_RHO * iplane] = rho.v;
-          w[I_UZ * iplane] = uz.v;
-          w[I_UR * iplane] = ur.v;
+        if constexpr (MODE == 3) {
+          double* w = inter + o;
+          if (role == 0) {
+            w[I_SZ * iplane] = unscale(sz, 36.0).v;
+            w[I_SR * iplane] = unscale(sr, 36.0).v;
+            w[I_PSI * iplane] = psi.v;
+          }
+          if (role == 1 % ROLES) {
+            w[I_DR * iplane] = unscale(dr0, 36.0).v;
+            w[I_DRR * iplane] = unscale(Drr, 1296.0).v;
+            w[I_DZR * iplane] = unscale(Dzr, 144.0).v;
+          }
+          if (role == 2 % ROLES) {
+            w[I_RHO * iplane] = rho.v;
+            w[I_UZ * iplane] = uz.v;
+            w[I_UR * iplane] = ur.v;
+          }
+          if (role == 3 % ROLES) {
+            w[I_VZ * iplane] = (fma(Fz, q.tau, jz) * inv_rho).v;
+            w[I_VR * iplane] = (fma(Fr, q.tau, jr) * inv_rho).v;
+            w[I_FZ * iplane] = Fz.v;
+            w[I_FR * iplane] = Fr.v;
+          }
         }
-        if (role == 3 % ROLES) {
-          w[I_VZ * iplane] = (fma(Fz, q.tau, jz) * inv_rho).v;
-          w[I_VR * iplane] = (fma(Fr, q.tau, jr) * inv_rho).v;
-          w[I_FZ * iplane] = Fz.v;
-          w[I_FR * iplane] = Fr.v;
-        }
-      }
-      double* out = (MODE == 3 ? fstar : f) + o;
-      with_role<ROLES>(role, [&](auto R) {
-        collide(q, guo, gk, fv, rho, uz, ur, jz, jr, Fz, Fr, inv_rho, [&](int i, T v) {
-          if (role_of(i, ROLES) == R.value) out[i * plane] = v.v;
+        with_role<ROLES>(role, [&](auto R) {
+          T g[9];
+          collide(q, guo, gk, fv, rho, uz, ur, jz, jr, Fz, Fr, inv_rho, [&](int i, T v) {
+            if (role_of(i, ROLES) != R.value || (ROLES > 1 && i == 0)) return;
+            out[i * plane] = v.v;
+            g[i] = v;
+          });
+          if constexpr (ROLES > 1) {  // the sums that leave the rest population
+            constexpr int first[4] = {1, 2, 5, 6};
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+              if (p % ROLES == R.value) sX[(10 + p) * G::SITES + t] = g[first[p]] + g[first[p] + 2];
+          }
         });
-      });
+      }
+    }
+    if constexpr (ROLES > 1 && MODE != 1) {
+      __syncthreads();
+      const T* x = sX + 10 * G::SITES + t;
+      if (in && role == 0) out[0] = rest_of(rho, x[0], x[G::SITES], x[2 * G::SITES], x[3 * G::SITES]).v;
     }
   }
 }
