@@ -418,12 +418,14 @@ int amlbm_batch_init_all(amlbm_batch* b, const double* rho, const double* uz, co
  * amlbm_batch_init_all of any FP64 arrays that round to these values. */
 int amlbm_batch_init_all_f32(amlbm_batch* b, const float* rho, const float* uz, const float* ur);
 /* The diagnostics of every instance in one pass (one read-back launch, one
- * partial-sum launch, one final launch, one device-to-host copy): dp holds n
- * parameter sets (NULL: the defaults of amlbm_batch_diagnostics), out receives
- * n results, each equal to what amlbm_batch_diagnostics gives for that
- * instance.  Returns AMLBM_EUNSTABLE, after filling every output, if any
- * instance has a non-finite or non-positive density (the message names the
- * first).  Synchronises the batch stream. */
+ * partial-sum launch, one final launch, whose results go to page-locked host
+ * memory in place): dp holds n parameter sets (NULL: the defaults of
+ * amlbm_batch_diagnostics), out receives n results, each equal to what
+ * amlbm_batch_diagnostics gives for that instance.  (How the sums of an instance
+ * are grouped depends on the sites of its whole batch, so the same lattice in
+ * another batch can differ in the last bits.)  Returns AMLBM_EUNSTABLE, after
+ * filling every output, if any instance has a non-finite or non-positive density
+ * (the message names the first).  Synchronises the batch stream. */
 int amlbm_batch_diagnostics_all(amlbm_batch* b, const amlbm_diag_params* dp, amlbm_diag* out);
 /* Sites of all instances (the work of one batch timestep). */
 long long amlbm_batch_sites(const amlbm_batch* b);

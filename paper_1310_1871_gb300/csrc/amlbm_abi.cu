@@ -927,7 +927,7 @@ int diag_host(amlbm_batch* b, int k, const amlbm_diag_params* dp, amlbm_diag* ou
   double* part = reinterpret_cast<double*>(b->arena + b->L.diag_part);
   double* cols = reinterpret_cast<double*>(b->arena + b->L.diag_cols);
   double* res = reinterpret_cast<double*>(b->arena + b->L.diag_out);
-  const int nblk = amlbm::diag_blocks(d.Nz, d.Nr, (long long)d.Nz * d.Nr);
+  const int nblk = amlbm::diag_blocks(d.Nz, d.Nr, b->sites);  // as diag_all_host: the same sums
   Pin pin;
   double own[16], *h = reinterpret_cast<double*>(pin.p);  // written by the kernel in place
   const cudaError_t e = amlbm::launch_diag(b->storage, b->d_desc, k, d.Nz, d.Nr, b->parity, p.zc, p.R,

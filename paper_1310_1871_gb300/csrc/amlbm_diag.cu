@@ -125,7 +125,8 @@ __device__ void partial_block(const InstDesc& D, const DiagJob& J, int blk, doub
   const C* __restrict__ rho_o = static_cast<const C*>(D.rho_out);
   const C* __restrict__ uz_o = static_cast<const C*>(D.uz_out);
   const C* __restrict__ ur_o = static_cast<const C*>(D.ur_out);
-  // Each thread first adds its own few sites (one to four) in C, then the block
+  // Each thread first adds its own sites (one to four on lattices of at most 1,048,576
+  // sites, ceil(Nz Nr / 262,144) beyond: 128 on 8192 x 4096) in C, then the block
   // and the final pass reduce those per-thread sums in FP64: the FP32 forms then
   // need one FP64 conversion and addition per sum and thread, not per site.
   C tacc[NSUM] = {C(0), C(0), C(0), C(0), C(0), C(0), C(0), C(0)};
@@ -168,7 +169,7 @@ __device__ void partial_block(const InstDesc& D, const DiagJob& J, int blk, doub
       }
     }
   }
-  // The warp's sums (up to 128 sites) pairwise in C too, then FP64 across warps and blocks.
+  // The warp's 32 sums pairwise in C too, then FP64 across warps and blocks.
   const double sum = double(warp_sums(tacc));
   const C top = warp_max_t(tacc[NSUM - 1]);
   __shared__ double red[DIAG_WARPS][NSUM];
@@ -309,7 +310,9 @@ void diag_job_constants(DiagJob& J) {
 }
 
 // One site per thread while the pass (`sites` over all its lattices) has at most eight
-// blocks per SM, up to four beyond.
+// blocks per SM, then two, then four; more only where 1024 blocks a lattice (1,048,576
+// sites) are not enough for that.  A batch counts the sites of all its lattices for a pass
+// over one of them too, so that both passes add in the same order.
 int diag_blocks(int Nz, int Nr, long long sites) {
   const long long round = 8LL * 152 * DIAG_NT;
   const int N = Nz * Nr, each = DIAG_NT * (sites <= round ? 1 : sites <= 2 * round ? 2 : 4);
