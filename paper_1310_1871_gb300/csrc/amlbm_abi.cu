@@ -192,9 +192,18 @@ int resolve_shift(const amlbm_bc& bc);
 // 14.4, 768 x 256 16.0 / 14.5, three threads of 344,448 sites 22.2 / 20.6, 700 x 700 22.7 / 26.8),
 // else the fused schedule: two rounds of the row kernel's largest tiles (512 x 256: 10.5 us per step; the
 // persistent grid on 26 x 16 14.4), beyond that the persistent grid (1024 x 512: 28.7; rows 36).
-void pick_tile(int storage, const std::vector<amlbm_instance>& inst, int* sched, int* tz, int* tr) {
+//
+// want: the schedule a caller asked for without a tile (0: none, the library's choice).
+// Of the rules above each schedule takes its own: pair the strips or 64 x 24 tiles, fused
+// the rest, split of the FP32-arithmetic forms (never chosen) and the FP64 kernels of fused
+// and pair 32 x 8.
+void pick_tile(int storage, const std::vector<amlbm_instance>& inst, int want, int* sched, int* tz, int* tr) {
+  *sched = want;
+  *tz = 32;
+  *tr = 8;
   if (storage == AMLBM_STORE_F64) {
     static const struct { int tz, tr, least; } pref64[] = {{32, 16, 912}, {32, 8, 96}, {16, 8, 128}, {8, 4, 0}};
+    if (want == amlbm::SCHED_FUSED || want == amlbm::SCHED_PAIR) return;
     *sched = amlbm::SCHED_SPLIT;
     for (const auto& t : pref64) {
       *tz = t.tz;
@@ -202,11 +211,14 @@ void pick_tile(int storage, const std::vector<amlbm_instance>& inst, int* sched,
       if (count_tiles(inst, t.tz, t.tr) >= t.least) return;
     }
   }
-  *sched = amlbm::SCHED_FUSED;
-  *tz = amlbm::kRowWidth;
-  *tr = amlbm::row_height([&](int h) { return count_tiles(inst, amlbm::kRowWidth, h); });
-  if (*tr) return;
-  if (all_pair_ok(inst, storage == AMLBM_STORE_F32)) {
+  if (want == amlbm::SCHED_SPLIT) return;
+  if (want != amlbm::SCHED_PAIR) {
+    *sched = amlbm::SCHED_FUSED;
+    *tz = amlbm::kRowWidth;
+    *tr = amlbm::row_height([&](int h) { return count_tiles(inst, amlbm::kRowWidth, h); });
+    if (*tr) return;
+  }
+  if (want == amlbm::SCHED_PAIR || (!want && all_pair_ok(inst, storage == AMLBM_STORE_F32))) {
     *sched = amlbm::SCHED_PAIR;
     *tz = amlbm::kStripWidth;
     double units = 0.0;
@@ -222,11 +234,7 @@ void pick_tile(int storage, const std::vector<amlbm_instance>& inst, int* sched,
     }
     return;
   }
-  if (count_tiles(inst, amlbm::kRowWidth, amlbm::kRowMaxRows) <= 4 * 152) {
-    *tr = amlbm::kRowMaxRows;
-    return;
-  }
-  *tr = 16;
+  *tr = count_tiles(inst, amlbm::kRowWidth, amlbm::kRowMaxRows) <= 4 * 152 ? amlbm::kRowMaxRows : 16;
 }
 
 // Shift code the kernels use: 0 none, 1 global rho_ref, 2 local (from psi),
@@ -505,16 +513,12 @@ int batch_build(const std::vector<amlbm_instance>& inst, const amlbm_tune* tune,
         if (bounded(I.bc))  // the FP64 kernels would take them; the documented choice is refused all the same
           return fail(AMLBM_EINVAL,
                       "the split schedule takes periodic lattices on the axis with the velocity shift only");
-    if (!tz && !tr) {
-      int s2;
-      pick_tile(storage, inst, &s2, &tz, &tr);
-      if (!amlbm::tile_supported(storage, sched, tz, tr)) { tz = 32; tr = 8; }
-    }
+    if (!tz && !tr) pick_tile(storage, inst, sched, &sched, &tz, &tr);
     if (!amlbm::tile_supported(storage, sched, tz, tr))
       return fail(AMLBM_EINVAL, "tile " + std::to_string(tz) + "x" + std::to_string(tr) +
                                     " is not compiled for this storage and schedule (see amlbm_tiles)");
   } else {
-    pick_tile(storage, inst, &sched, &tz, &tr);
+    pick_tile(storage, inst, 0, &sched, &tz, &tr);
   }
   amlbm_batch* b = new (std::nothrow) amlbm_batch();
   if (!b) return fail(AMLBM_ENOMEM, "host allocation failed");
