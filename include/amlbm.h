@@ -332,16 +332,19 @@ typedef struct amlbm_instance {
  * kernel writes u and u^eq per site, then a collide-stream kernel reads them with
  * a halo (less recomputation, 16 or 32 more bytes per site through L2); for FP64
  * the force kernel also collides, in place, and nearly nothing is recomputed: the
- * library's choice for every FP64 lattice, the bounded ones too, which a caller
- * cannot request it for.  PAIR:
+ * library's choice for every FP64 lattice.  A request for it takes periodic
+ * lattices on the axis with the velocity shift.  PAIR:
  * the fused update with two adjacent z-sites per thread (vector loads and
  * stores, stencil taps shared by the pair), on tiles, or for the FP32-arithmetic
  * forms with tile_z = 48 on strips: one warp marches over tile_r rows of 48
  * columns (a lattice of at most 64 columns is one strip); the library's own choice
- * for FP32 storage runs lattices of odd width on strips too.  A request for it takes periodic lattices on the
- * axis with an even Nz, a free-slip or no-slip outer wall, the source at the
- * departure site (AMLBM_SRC_LOCAL) and either forcing, and 9 x pitch x Nr below
- * 2^31 elements.  All three give bit-identical states. */
+ * for FP32 storage runs lattices of odd width on strips too.  A request for it takes
+ * periodic lattices on the axis with an even Nz, a free-slip or no-slip outer wall,
+ * the source at the departure site (AMLBM_SRC_LOCAL) and either forcing, and
+ * 9 x pitch x Nr below 2^31 elements.  Beyond these, exactly the schedule and tile
+ * that are the library's own choice for the instances (amlbm_batch_config of a batch
+ * made without a request) can be requested for them.  All three give bit-identical
+ * states. */
 #define AMLBM_SCHED_AUTO 0
 #define AMLBM_SCHED_FUSED 1
 #define AMLBM_SCHED_SPLIT 2
@@ -371,11 +374,13 @@ typedef struct amlbm_tune_result {
 
 /* Autotuner (no counterpart in the paper, which fixes no launch shape): for the
  * n instances (all with inst[0].bc.storage) it creates a temporary batch for
- * every compiled (schedule, tile) pair, sets a resting drop on every lattice,
- * runs 3 warm-up and 3 x `steps` timed timesteps on cuda_stream, and writes the
- * fastest pair to *best (graph_chunk 0; a candidate within 0.5 % of an earlier
- * one, in schedule and amlbm_tiles order, does not replace it) and, when results
- * is not NULL, up to cap candidates with their timings.  Every candidate computes the same state.
+ * every compiled (schedule, tile) pair a caller may request for them, and for the
+ * library's own choice where it is none of those, sets a resting drop on every
+ * lattice, runs 3 warm-up and 3 x `steps` timed timesteps on cuda_stream, and writes
+ * the fastest to *best (graph_chunk 0; a candidate within 0.5 % of an earlier one, in
+ * schedule and amlbm_tiles order, the library's own choice last, does not replace
+ * it) and, when results is not NULL, up to cap candidates with their timings.  Every
+ * candidate computes the same state.
  * Allocates and frees device memory for each candidate (it is not capturable)
  * and synchronises the stream.  Returns the number of candidates timed (> 0)
  * or a negative status. */

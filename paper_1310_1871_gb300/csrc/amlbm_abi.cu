@@ -88,8 +88,9 @@ amlbm_bc default_bc() {
   return b;
 }
 
-// A lattice with walls in z, an inlet or an outlet, or with the Guo forcing:
-// the fused schedule only.
+// A lattice with walls in z, an inlet or an outlet, or with the Guo forcing: a caller cannot
+// request the split schedule for it (the FP64 form's kernels take it all the same, as the
+// library's own choice).
 bool bounded(const amlbm_bc& bc) {
   return bc.z_bc != AMLBM_Z_PERIODIC || bc.r_lo != AMLBM_RLO_AXIS || bc.wall_r == AMLBM_WALL_OUTLET ||
          bc.forcing != AMLBM_FORCE_SHIFT;
@@ -504,15 +505,19 @@ int batch_build(const std::vector<amlbm_instance>& inst, const amlbm_tune* tune,
     sched = tune->schedule ? tune->schedule : (any_bounded ? AMLBM_SCHED_FUSED : AMLBM_SCHED_SPLIT);
     if (sched != AMLBM_SCHED_FUSED && sched != AMLBM_SCHED_SPLIT && sched != AMLBM_SCHED_PAIR)
       return fail(AMLBM_EINVAL, "bad schedule");
-    if (sched == AMLBM_SCHED_PAIR && !all_pair_ok(inst))
+    // what amlbm_batch_config reports of a batch made without a request is taken back
+    auto own_choice = [&] {
+      int s, z, r;
+      pick_tile(storage, inst, 0, &s, &z, &r);
+      return s == sched && z == tz && r == tr;
+    };
+    if (sched == AMLBM_SCHED_PAIR && !all_pair_ok(inst) && !own_choice())
       return fail(AMLBM_EINVAL,
                   "the pair schedule takes periodic lattices on the axis with an even Nz, a free-slip or "
                   "no-slip wall and the source at the departure site");
-    if (sched == AMLBM_SCHED_SPLIT)
-      for (const auto& I : inst)
-        if (bounded(I.bc))  // the FP64 kernels would take them; the documented choice is refused all the same
-          return fail(AMLBM_EINVAL,
-                      "the split schedule takes periodic lattices on the axis with the velocity shift only");
+    if (sched == AMLBM_SCHED_SPLIT && any_bounded && !own_choice())
+      return fail(AMLBM_EINVAL,
+                  "the split schedule takes periodic lattices on the axis with the velocity shift only");
     if (!tz && !tr) pick_tile(storage, inst, sched, &sched, &tz, &tr);
     if (!amlbm::tile_supported(storage, sched, tz, tr))
       return fail(AMLBM_EINVAL, "tile " + std::to_string(tz) + "x" + std::to_string(tr) +
@@ -953,7 +958,7 @@ int diag_host(amlbm_batch* b, int k, const amlbm_diag_params* dp, amlbm_diag* ou
 extern "C" {
 
 const char* amlbm_last_error(void) { return g_err.c_str(); }
-const char* amlbm_version(void) { return "amlbm 0.3 (sm_103a)"; }
+const char* amlbm_version(void) { return "amlbm 0.4 (sm_103a)"; }
 
 int amlbm_tiles(int storage, int schedule, int* tz, int* tr, int cap) {
   return amlbm::tile_list(storage, schedule, tz, tr, cap);
@@ -1206,6 +1211,17 @@ int ctx_info(amlbm_ctx* c, CtxInfo* out) {
   out->parity = b->parity;
   out->steps = b->steps[0];
   out->stream = b->stream;
+  return AMLBM_OK;
+}
+
+int library_choice(int n, const amlbm_instance* inst, amlbm_tune* t) {
+  std::vector<amlbm_instance> v(inst, inst + n);
+  for (int i = 0; i < n; ++i) {
+    const int rc = validate(v[i], i);
+    if (rc) return rc;
+  }
+  std::memset(t, 0, sizeof(*t));
+  pick_tile(v[0].bc.storage, v, 0, &t->schedule, &t->tile_z, &t->tile_r);
   return AMLBM_OK;
 }
 

@@ -241,6 +241,9 @@ int ctx_info(amlbm_ctx* ctx, CtxInfo* out);
 // Enqueue the read-back kernel (rho and u of the current state into the
 // context's own buffers).
 int ctx_readback(amlbm_ctx* ctx);
+// The schedule and tile that amlbm_batch_create takes for these instances when the caller
+// gives none (graph_chunk 0); an error status for instances it would refuse.
+int library_choice(int n, const amlbm_instance* inst, amlbm_tune* t);
 // Record a message for amlbm_last_error() and return code.
 int set_error(int code, const std::string& msg);
 // Shared by the diagnostics entry points (amlbm_abi.cu): the amlbm_diag of a

@@ -34,3 +34,17 @@ def test_what_a_schedule_cannot_take_is_still_refused(storage, kw):
             assert create(shapes, storage, schedule, **extra, **kw) == amlbm.EINVAL
     assert create([(63, 32)], storage, "pair", **kw) == amlbm.EINVAL
     assert create([(64, 32)], storage, "fused", (128, 8), **kw) == amlbm.EINVAL
+
+
+def test_own_choice_can_be_requested():
+    """The FP64 kernels on a bounded lattice, strips on an odd width: refused as a request
+    unless they are what the library takes by itself."""
+    discs = dict(z_bc="noslip", r_lo="inlet", r_off=9.0, wall="outlet")
+    for kw in (discs, dict(forcing="guo")):
+        assert create([(32, 111)], "f64", "split", (8, 4), **kw) == amlbm.ENOMEM
+        assert create([(32, 111)], "f64", "split", (16, 8), **kw) == amlbm.EINVAL
+        assert create([(32, 111)], "f64", "split", **kw) == amlbm.EINVAL
+        assert create([(32, 111)], "f32", "split", (32, 8), **kw) == amlbm.EINVAL
+    own = [create([(1025, 512)], "f32", "pair", (48, h)) == amlbm.ENOMEM for h in range(2, 130, 4)]
+    assert sum(own) == 1
+    assert all(create([(1025, 512)], "f16", "pair", (48, h)) == amlbm.EINVAL for h in range(2, 130, 4))
