@@ -414,7 +414,13 @@ namespace {
 // block to itself and gives it back when it has synchronised.  Measured, us: 128 bytes
 // launch to host 14.4 by a copy to pageable memory, 9.3 in place; three fields of 28,800
 // FP32 sites 33 by three copies to pageable memory, 14.5 by one copy here.
-constexpr size_t kPinBytes = 1 << 20, kPinKept = 8;
+//
+// A read of FP64 fields needs no widening, so above kDirectBytes in all it is copied straight
+// into the caller's arrays.  Measured, us a read of n sites through a block / straight to
+// pageable / to page-locked memory: 4,800 33 / 45 / 29; 8,192 38 / 45 / 29; 12,800 45 / 46 /
+// 30; 32,768 76 / 49 / 32; 524,288 1087 / 184 / 167.  FP32 is widened on the way: through blocks
+// at every size (32,768 47, 524,288 574; by whole copies and then the widening 75 and 634).
+constexpr size_t kPinBytes = 1 << 20, kPinKept = 8, kDirectBytes = 240 << 10;
 std::mutex g_pin_mu;
 std::vector<char*> g_pin_free;
 
@@ -762,9 +768,15 @@ int read_host(amlbm_batch* b, int k, double* rho, double* uz, double* ur, double
   if (rho || uz || ur) {
     rc = macro_for(b, k);
     if (rc) return rc;
-    // the read-back holds the compute type, FP32 to be widened: through the batch's
-    // page-locked block, all three fields in one copy where they fit
+    // the read-back holds the compute type, FP32 to be widened: through a page-locked
+    // block, all three fields in one copy where they fit; large FP64 ones straight
     const size_t es = compute_bytes(b->storage);
+    if (es == 8 && 3 * N * es > kDirectBytes) {
+      for (int q = 0; q < 3; ++q)
+        if (dst[q]) AMLBM_CK(cudaMemcpyAsync(dst[q], src[q], N * es, cudaMemcpyDeviceToHost, b->stream));
+      AMLBM_CK(cudaStreamSynchronize(b->stream));
+      return AMLBM_OK;
+    }
     std::vector<char> pageable;
     Pin pin;
     char* stage = pin.p;
