@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(Geo64<BZ, BR>::NT) f64_force(const InstDesc* _
       constexpr int NS = G::SITES;
       T* x = sX + t;
 #pragma unroll
-      for (int i = 0; i < 9; ++i) fv[i] = T{f[i * plane + o]};
+      for (int i = 0; i < 9; ++i) fv[i] = in ? T{f[i * plane + o]} : lit<T>(0.0);
       if (role == 0) {
         sc_sums(p, G::PZ, sz, sr);
         const T gpsi = psi * q.negG36;
