@@ -73,7 +73,7 @@ __device__ __forceinline__ unsigned long long bits_min(unsigned long long x) {
 // when no row is.  r0 is the radius of row 0.  Rows are scanned 32 at a time, the loads of
 // four such groups in flight together.
 template <class C>
-__device__ double col_radius_warp(const C* __restrict__ rho, int Nz, int Nr, int k, double mid, double r0) {
+__device__ double col_radius_warp(const C* rho, int Nz, int Nr, int k, double mid, double r0) {
   const C midc = C(mid);
   const int lane = threadIdx.x & 31;
   for (int j4 = 0; j4 < Nr; j4 += 128) {
@@ -122,9 +122,9 @@ __device__ void partial_block(const InstDesc& D, const DiagJob& J, int blk, doub
   const C two_pi = C(2.0 * 3.14159265358979323846);
   const C inv_dl = C(J.inv_dl), rho_v = C(J.rho_v), zc = C(J.zc);
   const C r0 = sizeof(C) == 8 ? C(D.k64[K_R0]) : C(D.k32[K_R0]);
-  const C* __restrict__ rho_o = static_cast<const C*>(D.rho_out);
-  const C* __restrict__ uz_o = static_cast<const C*>(D.uz_out);
-  const C* __restrict__ ur_o = static_cast<const C*>(D.ur_out);
+  const C* rho_o = static_cast<const C*>(D.rho_out);
+  const C* uz_o = static_cast<const C*>(D.uz_out);
+  const C* ur_o = static_cast<const C*>(D.ur_out);
   // Each thread first adds its own sites (one to four on lattices of at most 1,048,576
   // sites, ceil(Nz Nr / 262,144) beyond: 128 on 8192 x 4096) in C, then the block
   // and the final pass reduce those per-thread sums in FP64: the FP32 forms then

@@ -1,7 +1,10 @@
 // Programmatic dependent launch (sm_90 and later): a kernel launched with launch_pdl
 // may start while the kernel before it on the stream still runs.  It may read what
-// lattice creation wrote before pdl_wait(), everything else only after it: the wait
-// returns when the kernels before it have finished and their writes are visible.
+// was complete before that kernel was launched (descriptors and tile lists: whoever uploads
+// them synchronises before the first launch) before pdl_wait(), everything else only after
+// it: the wait returns when the kernels before it have finished and their writes are visible.
+// What they write is not read through const __restrict__ kernel arguments or __ldg, which
+// promise data that stays the same while this kernel runs.
 // pdl_trigger() lets the next kernel of the stream start early in turn; its blocks
 // take only room that this kernel's blocks, all placed by then, leave free.
 //

@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(Geo64<BZ, BR>::NT) f64_force(const InstDesc* _
   const int k0 = (l % tz) * BZ, j0 = (l / tz) * BR;
   const size_t plane = (size_t)P * Nr;
   double* f = static_cast<double*>(D.f[parity]);
-  const double* __restrict__ psin = static_cast<const double*>(D.psi[parity]);
+  const double* psin = static_cast<const double*>(D.psi[parity]);
   const bool ax = D.axisym != 0, zw = D.zbc == AMLBM_Z_NOSLIP;
   const bool inl = D.rlo == AMLBM_RLO_INLET, outl = D.wall == AMLBM_WALL_OUTLET;
   const bool guo = D.forcing == AMLBM_FORCE_GUO;
@@ -287,7 +287,7 @@ template <int BZ, int BR, int MODE>
 __global__ void __launch_bounds__(Geo64<BZ, BR>::NT) f64_stream(const InstDesc* __restrict__ descs,
                                                                const int* __restrict__ tile_inst, int parity,
                                                                double* __restrict__ inter, size_t iplane,
-                                                               const double* __restrict__ fstar,
+                                                               const double* fstar,
                                                                int* __restrict__ ctr) {
   using T = D1;
   using G = Geo64<BZ, BR>;
@@ -304,8 +304,8 @@ __global__ void __launch_bounds__(Geo64<BZ, BR>::NT) f64_stream(const InstDesc* 
   const int l = tile - D.tile_base;
   const int k0 = (l % D.tiles_z) * BZ, j0 = (l / D.tiles_z) * BR;
   const size_t plane = (size_t)P * Nr;
-  const double* __restrict__ fs = MODE == 3 ? fstar : static_cast<const double*>(D.f[parity]);
-  const double* __restrict__ uv = static_cast<const double*>(D.uv);
+  const double* fs = MODE == 3 ? fstar : static_cast<const double*>(D.f[parity]);
+  const double* uv = static_cast<const double*>(D.uv);
   const bool ax = D.axisym != 0, zw = D.zbc == AMLBM_Z_NOSLIP;
   const bool inl = D.rlo == AMLBM_RLO_INLET, outl = D.wall == AMLBM_WALL_OUTLET;
   const bool noslip = D.wall == AMLBM_WALL_NOSLIP, link = D.src == AMLBM_SRC_LINK;
