@@ -165,8 +165,10 @@ extern "C" int amlbm_flat_interface(double G, double tau, double rho0, int axisy
   }
   e = cudaMemcpyAsync(B.p[0], &d, sizeof(InstDesc), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(B.p[1], 0, ntiles * sizeof(int), s);
+  // both are read by the kernel before it waits for what is before it (amlbm_launch.cuh)
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e == cudaSuccess)
-    e = amlbm::launch_step_inter(storage, itz, itr, static_cast<const InstDesc*>(B.p[0]), 
+    e = amlbm::launch_step_inter(storage, itz, itr, static_cast<const InstDesc*>(B.p[0]),
                                  static_cast<const int*>(B.p[1]), ntiles, B.p[2], plane, d.f[0],
                                  s);  // that state is not needed any more
   if (e == cudaSuccess) {
