@@ -26,11 +26,12 @@
 // deterministic.
 //
 // Collision: with the moments M0 = sum W mu, M = sum W c mu, MM = sum W c c mu of the
-// gathered mu, the adjoint of f^eq is a quadratic form in u^eq: 57 operations instead of
-// nine separate terms (about 190).
+// gathered mu (less its value at rest, which takes the cancellation out of the tau part), the
+// adjoint of f^eq is a quadratic form in u^eq: 65 operations instead of nine separate terms
+// (about 190).
 //
 // Measured (GB300, ncu, one backward step, cold caches; the four kernels before): FP32,
-// 512 x 128: 21 us (45); FP64, 256 x 128: 36 us (68), 271 FP64 operations per site (543).
+// 512 x 128: 21 us (45); FP64, 256 x 128: 36 us (68), 279 FP64 operations per site (543).
 // A gradient of the differentiable drop, 512 x 128, T = 100, checkpoints every 10, FP32:
 // 2.5 ms (5.2; 2.8 with the forward steps on the persistent tiles); 256 x 128, T = 50, FP64: 3.8 ms (5.6).
 
@@ -89,12 +90,6 @@ struct Adj {
   C *rhob, *jzb, *jrb, *psib, *qz, *qr, *dzrb, *drrb, *drdb;  // adjoints, [Nr][P] each
   double *accG, *accT;
 };
-
-template <class C>
-__device__ __forceinline__ C feq_std(int i, C rho, C vz, C vr) {
-  const C cv = C(acz(i)) * vz + C(acr(i)) * vr;
-  return C(aw(i)) * rho * (C(1) + C(3) * cv + C(4.5) * cv * cv - C(1.5) * (vz * vz + vr * vr));
-}
 
 // mu_q at the lattice site (k, j): lambda where population q leaving it arrives
 // (Sec. II.E maps).
@@ -212,36 +207,38 @@ __global__ void __launch_bounds__(ATZ * BR) adj_local(Adj<C> A) {
   const C* I = A.inter + o;
   const C rho = I[I_RHO * A.plane], vz = I[I_VZ * A.plane], vr = I[I_VR * A.plane];
   const C uz = I[I_UZ * A.plane], ur = I[I_UR * A.plane];
-  // moments of mu, 9 times: M0, M_z, M_r, M_zz, M_zr, M_rr
-  const C pz = mu[1] + mu[3], pr = mu[2] + mu[4], ps = mu[5] + mu[7], pd = mu[6] + mu[8];
+  // moments of mu - mu_0, 9 times: M0, M_z, M_r, M_zz, M_zr, M_rr.  mu is nearly the same for
+  // all directions, and what is formed below depends on a constant mu only through
+  // sum mu f^eq = mu_0 rho: taken of mu itself, the tau part is a difference of two sums that
+  // agree to almost every bit, and term by term it keeps the rounding of f and of the weights
+  // times mu.  Against an 80-bit complex-step derivative of 85 random gradients (16 x 32 to
+  // 40 x 88, 8 to 50 steps), geometric mean of the relative error of dJ/dtau, term by term /
+  // from mu / from mu - mu_0: FP64 1.4e-13 / 1.2e-13 / 5.7e-15, FP32 3.2e-5 / 2.4e-5 / 3.5e-6.
+  const C Mz = first_z(mu), Mr = first_r(mu), mu0 = mu[0];
+  C dm[9];
+#pragma unroll
+  for (int q = 1; q < 9; ++q) dm[q] = mu[q] - mu0;
+  const C pz = dm[1] + dm[3], pr = dm[2] + dm[4], ps = dm[5] + dm[7], pd = dm[6] + dm[8];
   const C diag = C(0.25) * (ps + pd);
   const C Mzz = pz + diag, Mrr = pr + diag, Mzr = C(0.25) * (ps - pd);
-  const C M0 = C(4) * mu[0] + (pz + pr) + diag;
-  const C Mz = first_z(mu), Mr = first_r(mu);
+  const C M0 = (pz + pr) + diag;
   const C tz = vz * Mzz + vr * Mzr, tr = vz * Mzr + vr * Mrr;
   const C Aq = C(1) - C(1.5) * (vz * vz + vr * vr);
-  // sum mu f^eq / rho, and the adjoints of u^eq
+  // sum (mu - mu_0) f^eq / rho, and the adjoints of u^eq
   const C fe = C(1.0 / 9.0) * (Aq * M0 + C(4.5) * (vz * tz + vr * tr) + C(3) * (vz * Mz + vr * Mr));
-  // tau part, -omega^2 sum mu (f^eq - f).  In FP32 term by term: mu is nearly the same
-  // for all directions, so the sums of mu f^eq and mu f agree to almost every bit, and
-  // their difference would keep only rounding.
+  // tau part, -omega^2 sum (mu - mu_0) (f^eq - f): both sum to rho
   C tb = C(0);
-  if constexpr (sizeof(C) == 8) {
 #pragma unroll
-    for (int q = 0; q < 9; ++q) tb += mu[q] * A.f[q * A.plane + o];
-    tb -= rho * fe;
-  } else {
-#pragma unroll
-    for (int q = 0; q < 9; ++q) tb += mu[q] * (A.f[q * A.plane + o] - feq_std(q, rho, vz, vr));
-  }
+  for (int q = 1; q < 9; ++q) tb += dm[q] * A.f[q * A.plane + o];
+  tb -= rho * fe;
   tb *= A.omega * A.omega;
-  C rb = A.omega * fe;
+  C rb = A.omega * (mu0 + fe);
   const C com = A.omega * rho * C(1.0 / 3.0);
   const C vzb = com * (Mz + C(3) * tz - vz * M0), vrb = com * (Mr + C(3) * tr - vr * M0);
   C uzb = C(0), urb = C(0);
   const C irr = A.axisym ? s_ir[ty + 2] : C(0);
   if (A.axisym) {
-    const C Sb = C(1.0 / 9.0) * M0, Hzb = C(1.0 / 3.0) * Mz, Hrb = C(1.0 / 3.0) * Mr;
+    const C Sb = mu0 + C(1.0 / 9.0) * M0, Hzb = C(1.0 / 3.0) * Mz, Hrb = C(1.0 / 3.0) * Mr;
     const C d1r = I[I_G1 * A.plane] + I[I_G2 * A.plane], d3 = I[I_G3 * A.plane];
     const C muv = rho * cmu;
     // S = -rho u_r / r, H_z = (mu (g1 + g2) - rho u_r u_z) / r,
@@ -357,7 +354,10 @@ __global__ void __launch_bounds__(ATZ * BR) adj_psi(Adj<C> A) {
       pb += d1_t(seb + (ty + 2) * ATZ + tx, ATZ) * C(1.0 / 12.0);
       pb += iso_t(sdr + (ty + 2) * DZ + tx + 2, DZ) * C(1.0 / 36.0);
     }
-    // d psi / d rho = exp(-rho / rho0); in FP64 1 - psi / rho0 (an exp is 20 FP64 operations)
+    // d psi / d rho = exp(-rho / rho0); in FP64 1 - psi / rho0 (an exp is 20 FP64 operations),
+    // whose error is 2^-53 of psi / rho0 however small the derivative is: a rounding of rho_bar
+    // itself, to which it is added (gradients at rho up to 32 rho0 have the same error with
+    // either)
     C dpsi;
     if constexpr (sizeof(C) == 8) dpsi = C(1) - A.inter[I_PSI * A.plane + o] * A.inv_rho0;
     else dpsi = exp(-A.inter[I_RHO * A.plane + o] * A.inv_rho0);
