@@ -181,10 +181,9 @@ int resolve_shift(const amlbm_bc& bc);
 //
 // FP64: the two kernels of amlbm_step_split64.cu, on the largest tile that still keeps
 // the 152 SMs busy.  Measured (us per step on 8 x 4 / 16 x 8 / 32 x 8 / 32 x 16 tiles):
-// 64 x 32 9.2 / 14.4 / 21.1 / 36.0 (the recomputing kernels before: 38); 192 x 96 16.6 /
-// 14.7 / 21.2 / 35.8; 256 x 128 26.1 / 24.2 / 21.0 / 38.3; 512 x 256 90 / 68 / 68.0 / 66.5;
-// 1024 x 512 338 / 250 / 227 / 218 (before: 394); 330,400 sites in 25 lattices 217 / 168 /
-// 158.5 / 164.5.
+// 64 x 32 8.9 / 14.2 / 21.4 / 35.7 (the recomputing kernels before: 38); 192 x 96 18.2 /
+// 15.1 / 21.1 / 36.6; 256 x 128 26.6 / 24.5 / 21.4 / 36.8; 512 x 256 92 / 70 / 69.7 / 67.8;
+// 1024 x 512 345 / 256 / 233 / 224 (before: 394).
 //
 // FP32 arithmetic: the row kernel's tiles while they all run at once (row_height), then
 // the pair schedule's strips where every lattice allows them (pick_strip; with the

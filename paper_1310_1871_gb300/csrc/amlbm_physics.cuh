@@ -465,18 +465,18 @@ __device__ __forceinline__ void collide(const Par<T>& q, bool guo, T gk, const T
     const T quarter = lit<T>(0.25);
     const T qz = fma(ez, vz, a9), qr = fma(er, vr, a9);
     const T qs = fma(es, sv, a9), qd = fma(ed, dv, a9), ks = kz + kr, kd = kr - kz;
-    T g[9];
-    g[1] = fma(q.om1, f[1], qz + kz);
-    g[3] = fma(q.om1, f[3], qz - kz);
-    g[2] = fma(q.om1, f[2], qr + kr);
-    g[4] = fma(q.om1, f[4], qr - kr);
-    g[5] = fma(q.om1, f[5], (qs + ks) * quarter);
-    g[7] = fma(q.om1, f[7], (qs - ks) * quarter);
-    g[6] = fma(q.om1, f[6], (qd + kd) * quarter);
-    g[8] = fma(q.om1, f[8], (qd - kd) * quarter);
-    g[0] = rest_of(rho, g[1] + g[3], g[2] + g[4], g[5] + g[7], g[6] + g[8]);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) put(i, g[i]);
+    // each pair is put as it is formed: only the sums stay live
+    auto pair = [&](int a, T up, int b, T down) {
+      const T ga = fma(q.om1, f[a], up), gb = fma(q.om1, f[b], down);
+      put(a, ga);
+      put(b, gb);
+      return ga + gb;
+    };
+    const T pz = pair(1, qz + kz, 3, qz - kz);
+    const T pr = pair(2, qr + kr, 4, qr - kr);
+    const T ps = pair(5, (qs + ks) * quarter, 7, (qs - ks) * quarter);
+    const T pd = pair(6, (qd + kd) * quarter, 8, (qd - kd) * quarter);
+    put(0, rest_of(rho, pz, pr, ps, pd));
   } else {
     T fe[9];
     if (guo) {

@@ -23,9 +23,9 @@
 //
 // On small grids each kernel lets the next start as soon as it has begun to read
 // (pdl_trigger): its blocks then wait beside this one's with their index and row
-// constants ready.  us per step without / with it: 64 x 32 (64 blocks of 8 x 4) 10.7 / 9.2,
-// 128 x 64 (256) 12.7 / 11.0, 192 x 80 (480) 17.6 / 16.2, 256 x 128 (128 of 32 x 8) 22.7 / 21.0,
-// 384 x 200 (300) 37.1 / 35.8.  Beyond, the next kernel's blocks crowd onto the SMs that are
+// constants ready.  us per step without / with it: 64 x 32 (64 blocks of 8 x 4) 10.8 / 8.9,
+// 128 x 64 (256) 13.2 / 11.5, 192 x 80 (480) 17.8 / 16.6, 256 x 128 (128 of 32 x 8) 23.1 / 21.4,
+// 384 x 200 (300) 38.0 / 36.8.  Beyond, the next kernel's blocks crowd onto the SMs that are
 // free first: 192 x 120 (180 of 16 x 8) 23.6 / 27.3, 512 x 200 (400 of 32 x 8) 52.2 / 65.7.  The
 // adjoint's forward steps (MODE 3) never do: they run beside another stream, whose kernels
 // need the room (gradient of 256 x 128 over 50 steps 3.77 ms, with it 4.15).
@@ -56,6 +56,12 @@ struct Geo64 {
   static constexpr int ROLES = SITES >= 256 ? 1 : SITES >= 128 ? 2 : 4;
   static constexpr int NT = SITES * ROLES < 256 ? SITES * ROLES : 256;
   static_assert(SITES % 32 == 0 && (ROLES == 1 || NT == SITES * ROLES), "a role is whole warps");
+  // CTAs of f64_force per SM that its registers have to allow: on 512-site tiles three (79
+  // registers; left to itself the compiler takes 94).  On 256-site tiles it takes 64 by
+  // itself, which the early launch below needs: two CTAs of this kernel and two of the
+  // next fit an SM then.  With the nine populations held until the last is formed it takes
+  // 78, and 384 x 200 took 58.2 us a step, 304 x 160 45.7 (36.8 and 36.2).
+  static constexpr int kBlocks = SITES > 256 ? 3 : 0;
   // the largest grid that starts the next kernel early
   static constexpr unsigned kEarly = ROLES == 4 ? 512 : SITES == 256 ? 304 : 152;
   static constexpr int PZ = BZ + 8, PR = BR + 8;  // psi
@@ -106,7 +112,7 @@ __device__ __forceinline__ void with_role(int role, F&& body) {
 // state is left alone); MODE 3: the step's first half with the forward intermediates
 // for the adjoint (into `inter`), the collided populations going to `fstar`.
 template <int BZ, int BR, int MODE>
-__global__ void __launch_bounds__(Geo64<BZ, BR>::NT) f64_force(const InstDesc* __restrict__ descs,
+__global__ void __launch_bounds__(Geo64<BZ, BR>::NT, MODE == 0 ? Geo64<BZ, BR>::kBlocks : 0) f64_force(const InstDesc* __restrict__ descs,
                                                               const int* __restrict__ tile_inst, int toff,
                                                               int parity, double* __restrict__ inter, size_t iplane,
                                                               double* fstar) {
