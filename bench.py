@@ -367,6 +367,10 @@ def kernel_name(storage, sched, tile):
         return f"strip_step<{t}>, {tile[1]} rows", os.path.join(csrc, "amlbm_step_strip.cu")
     if sched == "pair":
         return f"pair_persistent<{t}, {tile[0]}, {tile[1]}>", os.path.join(csrc, "amlbm_step_pair.cu")
+    if sched == "fused" and tile[0] == 26 and tile[1] <= 10 and storage != "f64":
+        return f"row_kernel<{t}>, {tile[1]} rows", os.path.join(csrc, "amlbm_step_row.cu")
+    if sched == "split" and storage == "f64":
+        return f"f64_stream<{tile[0]}, {tile[1]}> + f64_force", os.path.join(csrc, "amlbm_step_split64.cu")
     if sched == "fused":
         return f"lbm_persistent<{t}, {tile[0]}, {tile[1]}>", os.path.join(csrc, "amlbm_step.cu")
     return f"stream_kernel<{t}, {tile[0]}, {tile[1]}> + force_kernel", os.path.join(csrc, "amlbm_step.cu")

@@ -186,12 +186,23 @@ int resolve_shift(const amlbm_bc& bc);
 // 1024 x 512 345 / 256 / 233 / 224 (before: 394).
 //
 // FP32 arithmetic: the row kernel's tiles while they all run at once (row_height), then
-// the pair schedule's strips where every lattice allows them (pick_strip; with the
-// equilibrium shift in 16 bits, whose codec makes a strip's rows longer, 64 x 24 tiles where
-// one or two rounds of them are faster: us per step on strips / tiles, FP16, 512 x 256 14.3 /
-// 14.4, 768 x 256 16.0 / 14.5, three threads of 344,448 sites 22.2 / 20.6, 700 x 700 22.7 / 26.8),
-// else the fused schedule: two rounds of the row kernel's largest tiles (512 x 256: 10.5 us per step; the
+// the pair schedule's strips where every lattice allows them (pick_strip), else the fused
+// schedule: two rounds of the row kernel's largest tiles (512 x 256: 10.5 us per step; the
 // persistent grid on 26 x 16 14.4), beyond that the persistent grid (1024 x 512: 28.7; rows 36).
+//
+// With the equilibrium shift in 16 bits, whose codec makes a strip's rows longer, 64 x 24 tiles
+// where one or two rounds of 152 of them are predicted to be faster.  The prediction is two
+// lines fitted to FP16 times: a step on tiles takes 14.4 us in one round and 20.5 in two
+// (8.2 + 6.2 rounds); on strips 1.7 + 1.05 times pick_strip's units, and 1.16 times that from
+// 608 strips on, where a sub-partition holds two of these longer ones; strips keep the ties
+// (0.95).  us per step, the chosen one first, FP16, then BF16: 512 x 256 strips 14.2 / 14.4,
+// 13.9 / 14.4; 768 x 256 tiles 14.4 / 15.7, 14.4 / 15.0; 600 x 500 strips 16.1 / 20.5, 15.3 / 20.5; 1024 x 400
+// tiles 20.5 / 22.6, 20.5 / 21.8; 700 x 700 strips 22.6 / 26.7, 21.6 / 26.7; three threads of 207 rows
+// tiles 20.5 / 22.3, 20.5 / 21.6; 8 lattices of 256 x 128 strips 16.2 / 20.5, 15.3 / 20.5.  A batch with
+// the shift on some lattices only runs the strips' branching form and gains more from tiles (one of
+// the three threads shifted: tiles 18.5 / 22.4, 18.5 / 22.5).  Of 19 FP16 and 19 BF16 batches
+// all shifted the choice is the slower by more than 4 % on one (2048 x 220, three rounds: 22.5 /
+// 20.5, 21.7 / 20.5), of 36 partly shifted ones on five (four times 16 drops of 137,920 sites, strips 16.1 .. 16.5 / 14.4).
 //
 // want: the schedule a caller asked for without a tile (0: none, the library's choice).
 // Of the rules above each schedule takes its own: pair the strips or 64 x 24 tiles, fused
@@ -224,7 +235,7 @@ void pick_tile(int storage, const std::vector<amlbm_instance>& inst, int want, i
     double units = 0.0;
     long long strips = 0;
     *tr = pick_strip(inst, &units, &strips);
-    bool shifted = false;
+    bool shifted = false;  // some lattice of the batch
     for (const auto& I : inst) shifted = shifted || resolve_shift(I.bc) == 3;
     const long long rounds = (count_tiles(inst, 64, 24) + 151) / 152;
     if (shifted && elem_bytes(storage) == 2 && rounds <= 2 &&

@@ -3,8 +3,8 @@
 // and later).  Each lane rounds as the scalar operation does, so a function evaluated
 // on F2 gives the bits of the same function on F1.  On GB300 a packed operation takes
 // the FP32 pipe as long as its two scalar ones (measured: 1.90 packed against 3.55
-// scalar warp instructions per clock and SM) but one issue slot, and issue slots are
-// what bounds the FP32 step.
+// scalar warp instructions per clock and SM) but one issue slot.  (What then bounds the
+// strips stands in amlbm_step_strip.cu.)
 //
 // A packed operand has no negation, so the specialisations below state the functions
 // of amlbm_physics.cuh with their negations moved into constants, differences and

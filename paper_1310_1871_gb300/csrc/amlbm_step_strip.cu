@@ -19,10 +19,13 @@
 // work).  A lattice of at most 64 columns is one strip without a halo: its lanes wrap
 // around the period.
 //
-// What bounds it: the FMA pipe's operand bandwidth.  A row is 224 packed operations; one
-// with three distinct operand pairs takes 3.2 clocks of its SM sub-partition, any other
-// 2.2 (measured), together about 580 of the 710 clocks a row takes of it with the two
-// warps that 220 registers a thread allow.  Three warps at 168 registers, with the delayed
+// What bounds it: the FMA pipe's operand bandwidth, with the two warps of a sub-partition
+// that 220 registers a thread allow.  A row is 224 packed operations; one with three distinct
+// operand pairs takes 3.2 clocks of its SM sub-partition, any other 2.2 (measured on loops of
+// them), together about 580 of the 710 clocks a row takes.  Counters of a step of 8192 x 1024
+// (ncu): FMA pipe 53 % and issue slots 48 % active, DRAM 59 %; per issued instruction a warp
+// waits 0.9 cycles at fixed latencies, 0.4 for shared memory and shuffles, 0.4 unselected.
+// Three warps at 168 registers, with the delayed
 // values in shared memory, were slower (8192 x 4096: 714 against 592 us).
 // Measured (GB300, FP32 storage, us per step; the 64 x 24 tile kernel before): the 64-drop
 // sweep of 835,240 sites 37.7 -> 21.5, eight threads of 3.6 M sites 119.7 -> 64.1,
