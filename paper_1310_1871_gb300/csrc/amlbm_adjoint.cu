@@ -33,7 +33,7 @@
 // Measured (GB300, ncu, one backward step, cold caches; the four kernels before): FP32,
 // 512 x 128: 21 us (45); FP64, 256 x 128: 36 us (68), 279 FP64 operations per site (543).
 // A gradient of the differentiable drop, 512 x 128, T = 100, checkpoints every 10, FP32:
-// 2.5 ms (5.2; 2.8 with the forward steps on the persistent tiles); 256 x 128, T = 50, FP64: 3.8 ms (5.6).
+// 2.5 ms (5.2; 2.8 with the forward steps on the persistent tiles); 256 x 128, T = 50, FP64: 3.9 ms (5.6).
 
 #include <cuda_runtime.h>
 
